@@ -45,6 +45,14 @@ constexpr int kChanAmg = 5;  // ... of the multigrid flow (B takes five dot prod
 __host__ __device__ constexpr int chan_count(bool amg) { return amg ? kChanAmg : kChan; }
 constexpr int kRedSlots = 3;
 constexpr int kMaxReq = 1024;
+// Tiles up to which a step's partials are summed by a warp an entry instead of
+// by the whole block entry after entry (arrive_and_finalize).  At 11 tiles the
+// block-wide sum took about 6 us in FP64 (it adds batches of 16 whether or not
+// there are that many tiles, on a pipe of one DADD a warp in 16 clocks); with
+// the tile butterflies above, FP64 reducing steps went from 9.5 to 7.5 us there
+// (2,562 rows), and B from 22 to 15 us at 28 tiles with four right-hand sides.
+// Above this count a lane's chain of additions is the longer one.
+constexpr int kFinWarpTiles = 512;
 constexpr long long kStageWaitLimit = 1ll << 24;  // polls of an mbarrier: far beyond any copy's landing time
 
 enum Phase : int { P_PRE_A = 0, P_A = 1, P_PRE_B = 2, P_B = 3, P_C = 4, P_COUNT = 5 };
@@ -211,46 +219,6 @@ __device__ __forceinline__ void c_row_f64(const Prob& P, int64_t r, const RhsSta
     }
 }
 
-// Warp totals of E F2 values a lane (E a power of two, at most 32) with a
-// fraction of the shuffles of E separate butterflies.  At each of the first
-// log2 E offsets (16, 8, ...) a lane keeps half of its values -- the upper
-// half if its bit at that offset is set -- and adds the partner's copy of
-// them; the remaining offsets add the one value left.  Every value is summed
-// in exactly the pairs and order of a plain xor butterfly over offsets 16, 8,
-// 4, 2, 1 (f2_add is commutative), so the totals are those of E separate
-// butterflies, bit for bit.  Returns the total of channel `chan` (set here)
-// that this lane ends with; lanes L with L % (32 / E) == 0 hold channels
-// 0 .. E-1 once each.
-template <int E>
-__device__ __forceinline__ F2 warp_sum_f2_multi(F2 (&v)[E], int lane, int& chan) {
-    static_assert(E >= 1 && E <= 32 && (E & (E - 1)) == 0, "a power of two, at most 32 values");
-    chan = 0;
-#pragma unroll
-    for (int t = 0; t < 5; t++) {
-        const int o = 16 >> t;
-        const int h = E >> (t + 1);  // values kept after this offset (0: one value left)
-        if (h >= 1) {
-            const bool up = (lane & o) != 0;
-#pragma unroll
-            for (int j = 0; j < (h >= 1 ? h : 1); j++) {
-                const F2 send = up ? v[j] : v[j + h];
-                const F2 keep = up ? v[j + h] : v[j];
-                F2 recv;
-                recv.hi = __shfl_xor_sync(0xffffffffu, send.hi, o);
-                recv.lo = __shfl_xor_sync(0xffffffffu, send.lo, o);
-                v[j] = f2_add(keep, recv);
-            }
-            if (up) chan += h;
-        } else {
-            F2 w;
-            w.hi = __shfl_xor_sync(0xffffffffu, v[0].hi, o);
-            w.lo = __shfl_xor_sync(0xffffffffu, v[0].lo, o);
-            v[0] = f2_add(v[0], w);
-        }
-    }
-    return v[0];
-}
-
 __host__ __device__ constexpr int pow2_at_least(int x) { return x <= 1 ? 1 : 2 * pow2_at_least((x + 1) / 2); }
 
 // Tile partials and their sums: F2 (double-float on the FP32 pipe) in the
@@ -301,50 +269,84 @@ __device__ __forceinline__ F2 part_load(const F2* p) {
 }
 __device__ __forceinline__ double part_load(const double* p) { return __ldcg(p); }
 
+__device__ __forceinline__ F2 part_shfl_xor(F2 v, int o) {
+    F2 w;
+    w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+    w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+    return w;
+}
+__device__ __forceinline__ double part_shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+
+// Warp totals of E values a lane (E a power of two, at most 32) with a
+// fraction of the shuffles and additions of E separate butterflies.  At each
+// of the first log2 E offsets (16, 8, ...) a lane keeps half of its values --
+// the upper half if its bit at that offset is set -- and adds the partner's
+// copy of them; the remaining offsets add the one value left.  Every value is
+// summed in exactly the pairs and order of a plain xor butterfly over offsets
+// 16, 8, 4, 2, 1 (additions commute), so the totals are those of E separate
+// butterflies, bit for bit.  Returns the total of value `chan` (set here)
+// that this lane ends with; lanes L with L % (32 / E) == 0 hold values
+// 0 .. E-1 once each.
+template <int E, typename PT>
+__device__ __forceinline__ PT warp_sum_multi(PT (&v)[E], int lane, int& chan) {
+    static_assert(E >= 1 && E <= 32 && (E & (E - 1)) == 0, "a power of two, at most 32 values");
+    chan = 0;
+#pragma unroll
+    for (int t = 0; t < 5; t++) {
+        const int o = 16 >> t;
+        const int h = E >> (t + 1);  // values kept after this offset (0: one value left)
+        if (h >= 1) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int j = 0; j < (h >= 1 ? h : 1); j++) {
+                const PT send = up ? v[j] : v[j + h];
+                const PT keep = up ? v[j + h] : v[j];
+                v[j] = part_add(keep, part_shfl_xor(send, o));
+            }
+            if (up) chan += h;
+        } else {
+            v[0] = part_add(v[0], part_shfl_xor(v[0], o));
+        }
+    }
+    return v[0];
+}
+
 // A warp's partials of its slice of a tile, channels 0 .. NCH-1 of every
-// right-hand side, into out[ch * QT + q]: the FP32 (F2) products summed over
-// the warp, plus the FP64 ones where there are any (`with64`).
+// right-hand side, into out[ch * QT + q]: in the FP32 flow the F2 products
+// summed over the warp, plus the FP64 ones where there are any (`with64`); in
+// the FP64 flow the FP64 ones.  The values go through the shared butterfly at
+// most 32 at a time.  In FP64 that is what bounds the step on a small system:
+// a DADD takes the SM's FP64 pipe 16 clocks a warp, so 5 channels in separate
+// butterflies (25 DADDs a warp, 9 here) held a tile's 8 warps for 1.5 us, and
+// 8 right-hand sides (200 against about 45) for 12 us.
 template <bool MIXED, int QT, int NC, int NCH>
 __device__ __forceinline__ void tile_partials(const F2 (&af)[NC][QT], const double (&ad)[NC][QT], bool with64,
                                               int lane, Part<MIXED>* out) {
-    using PT = Part<MIXED>;
-    constexpr int E = pow2_at_least(NCH * QT);
-    double w64[NCH * QT];
-#pragma unroll
-    for (int e = 0; e < NCH * QT; e++) w64[e] = with64 ? warp_sum(ad[e / QT][e % QT]) : 0.0;
-    if constexpr (MIXED && E > 32) {  // more values than lanes: one butterfly each
-#pragma unroll
-        for (int e = 0; e < NCH * QT; e++) {
-            F2 x = warp_sum_f2(af[e / QT][e % QT]);
-            if (with64) x = f2_add(x, part_from<F2>(w64[e]));
-            if (lane == 0) out[e] = x;
-        }
-    } else if constexpr (MIXED) {
-        constexpr int E32 = E > 32 ? 32 : E;
-        F2 v[E32];
-#pragma unroll
-        for (int e = 0; e < E32; e++) {
-            v[e].hi = 0.0f;
-            v[e].lo = 0.0f;
-            if (e < NCH * QT) v[e] = af[e / QT][e % QT];
-        }
+    constexpr int N = NCH * QT;
+    auto group = [&](auto width, int e0) {  // values e0 .. e0 + E - 1 (those past N are zeros)
+        constexpr int E = decltype(width)::value;
         int chan;
-        const F2 tot = warp_sum_f2_multi<E32>(v, lane, chan);
-        if ((lane & (32 / E32 - 1)) == 0 && chan < NCH * QT) {
-            F2 x = tot;
-            if (with64) {
-                double w = 0.0;
+        double tot64 = 0.0;
+        if (!MIXED || with64) {
+            double v[E];
 #pragma unroll
-                for (int e = 0; e < NCH * QT; e++)
-                    if (e == chan) w = w64[e];
-                x = f2_add(x, part_from<F2>(w));
-            }
-            out[chan] = x;
+            for (int e = 0; e < E; e++) v[e] = e0 + e < N ? ad[(e0 + e) / QT][(e0 + e) % QT] : 0.0;
+            tot64 = warp_sum_multi<E>(v, lane, chan);
         }
-    } else if (lane == 0) {
+        Part<MIXED> tot = part_from<Part<MIXED>>(tot64);
+        if constexpr (MIXED) {
+            F2 v[E];
 #pragma unroll
-        for (int e = 0; e < NCH * QT; e++) out[e] = part_from<PT>(w64[e]);
-    }
+            for (int e = 0; e < E; e++) v[e] = e0 + e < N ? af[(e0 + e) / QT][(e0 + e) % QT] : part_zero<F2>();
+            const F2 t = warp_sum_multi<E>(v, lane, chan);
+            tot = with64 ? f2_add(t, tot) : t;
+        }
+        if ((lane & (32 / E - 1)) == 0 && e0 + chan < N) out[e0 + chan] = tot;
+    };
+    constexpr int kHead = N > 32 ? 32 : pow2_at_least(N);
+    group(std::integral_constant<int, kHead>{}, 0);
+    if constexpr (N > 32) group(std::integral_constant<int, pow2_at_least(N - 32)>{}, 32);
+    static_assert(N <= 64, "two groups hold every channel of every right-hand side");
 }
 
 // Per-warp staging of operator slices.  A slice -- 32 rows' k column slots
@@ -976,7 +978,44 @@ __device__ __forceinline__ void arrive_and_finalize(const Prob& P, int ph, int s
         *last = lst;
     }
     __syncthreads();
-    if (*last) {
+    if (*last && P.nchunk <= kFinWarpTiles) {
+        // few tiles: a warp an entry (channel, right-hand side), tiles across its lanes
+        constexpr int kPerWarp = (NC * QT + kThreads / 32 - 1) / (kThreads / 32);
+        constexpr int kEnt = kPerWarp > 4 ? 4 : kPerWarp;  // entries a warp takes at once
+        constexpr int kDeep = kEnt >= 4 ? 2 : 4;  // tiles of an entry in flight a lane
+        const int nchunk = P.nchunk, Q = P.Q, E = nch * Q;
+        const PT* part = static_cast<const PT*>(P.part) + (int64_t)slot * NC * nchunk * Q;
+        for (int e0 = wid; e0 < E; e0 += kEnt * (kThreads / 32)) {  // warp-uniform
+            PT acc[kEnt];
+#pragma unroll
+            for (int u = 0; u < kEnt; u++) acc[u] = part_zero<PT>();
+            for (int l0 = lane; l0 - lane < nchunk; l0 += 32 * kDeep) {
+                PT v[kEnt][kDeep];
+#pragma unroll
+                for (int u = 0; u < kEnt; u++) {
+                    const int e = e0 + u * (kThreads / 32);
+#pragma unroll
+                    for (int d = 0; d < kDeep; d++) {
+                        const int l = l0 + 32 * d;
+                        v[u][d] = e < E && l < nchunk ? part_load(part + ((int64_t)(e / Q) * nchunk + l) * Q + e % Q)
+                                                      : part_zero<PT>();
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kEnt; u++)
+#pragma unroll
+                    for (int d = 0; d < kDeep; d++)
+                        if (l0 - lane + 32 * d < nchunk) acc[u] = part_add(acc[u], v[u][d]);
+            }
+#pragma unroll
+            for (int u = 0; u < kEnt; u++) {
+                const int e = e0 + u * (kThreads / 32);
+                if (e >= E) break;  // warp-uniform
+                const PT t = part_warp_sum(acc[u]);
+                if (lane == 0) tot[(e / Q) * QT + e % Q] = part_value(t);
+            }
+        }
+    } else if (*last) {
         constexpr int kFinBatch = (QT == 1 && !MIXED) ? 16 : 8;
         const int nchunk = P.nchunk, Q = P.Q;
         // two channels (or right-hand sides) at a time: 2 x kFinBatch loads in flight
@@ -1024,6 +1063,8 @@ __device__ __forceinline__ void arrive_and_finalize(const Prob& P, int ph, int s
             tot[tid] = part_value(part_add(part_add(part_add(f[0], f[W]), part_add(f[2 * W], f[3 * W])),
                                            part_add(part_add(f[4 * W], f[5 * W]), part_add(f[6 * W], f[7 * W]))));
         }
+    }
+    if (*last) {
         __syncthreads();
         if (tid < P.Q) {
             RhsState T = S[tid];
