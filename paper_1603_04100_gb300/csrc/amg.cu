@@ -516,15 +516,12 @@ __global__ void k_vcoarse(const AmgHeader* __restrict__ Hp, const double* __rest
     const int m = H.nlev - 1;
     const int64_t rho = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kWarp;
     if (rho >= H.nc) return;  // warp-uniform
-    for (int q = 0; q < Q; q++) {
-        float x;
-        if (m == 0) x = coarse_row(H, rho, [&](int64_t c) { return (float)b0[c * Q + q]; });
-        else x = coarse_row(H, rho, [&](int64_t c) { return V.b[m][c * Q + q]; });
-        if (lane_id() == 0) {
-            if (m == 0) x0[rho * Q + q] = (double)x;
-            else V.x[m][rho * Q + q] = x;
-        }
-    }
+    auto store = [&](int q, float x) {
+        if (m == 0) x0[rho * Q + q] = (double)x;
+        else V.x[m][rho * Q + q] = x;
+    };
+    if (m == 0) coarse_rows<8>(H, rho, b0, Q, store);
+    else coarse_rows<8>(H, rho, V.b[m], Q, store);
 }
 
 __global__ void __launch_bounds__(kApplyThreads) k_vup(const AmgHeader* __restrict__ Hp, int l, double* x0, int Q,

@@ -120,6 +120,50 @@ __device__ __forceinline__ F2 warp_sum_f2(F2 v) {
 
 __device__ __forceinline__ double f2_to_double(F2 v) { return (double)v.hi + (double)v.lo; }
 
+__device__ __forceinline__ F2 part_add(F2 a, F2 b) { return f2_add(a, b); }
+__device__ __forceinline__ double part_add(double a, double b) { return a + b; }
+__device__ __forceinline__ F2 part_shfl_xor(F2 v, int o) {
+    F2 w;
+    w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+    w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+    return w;
+}
+__device__ __forceinline__ double part_shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+
+// Warp totals of E values a lane (E a power of two, at most 32) with a
+// fraction of the shuffles and additions of E separate butterflies.  At each
+// of the first log2 E offsets (16, 8, ...) a lane keeps half of its values --
+// the upper half if its bit at that offset is set -- and adds the partner's
+// copy of them; the remaining offsets add the one value left.  Every value is
+// summed in exactly the pairs and order of a plain xor butterfly over offsets
+// 16, 8, 4, 2, 1 (additions commute), so the totals are those of E separate
+// butterflies, bit for bit.  Returns the total of value `chan` (set here)
+// that this lane ends with; lanes L with L % (32 / E) == 0 hold values
+// 0 .. E-1 once each.
+template <int E, typename PT>
+__device__ __forceinline__ PT warp_sum_multi(PT (&v)[E], int lane, int& chan) {
+    static_assert(E >= 1 && E <= 32 && (E & (E - 1)) == 0, "a power of two, at most 32 values");
+    chan = 0;
+#pragma unroll
+    for (int t = 0; t < 5; t++) {
+        const int o = 16 >> t;
+        const int h = E >> (t + 1);  // values kept after this offset (0: one value left)
+        if (h >= 1) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int j = 0; j < (h >= 1 ? h : 1); j++) {
+                const PT send = up ? v[j] : v[j + h];
+                const PT keep = up ? v[j + h] : v[j];
+                v[j] = part_add(keep, part_shfl_xor(send, o));
+            }
+            if (up) chan += h;
+        } else {
+            v[0] = part_add(v[0], part_shfl_xor(v[0], o));
+        }
+    }
+    return v[0];
+}
+
 __device__ __forceinline__ uint64_t shfl_u64(uint64_t v, int src) {
     return __shfl_sync(0xffffffffu, v, src);
 }

@@ -71,6 +71,9 @@ struct RhsState {
     int pending;     // multigrid flow: the last step's x += alpha ph + omega sh is still to apply
 };
 
+// Right-hand sides of the request (or group) in a kernel of width QT.
+#define MVGD_NQ(P) (QT == 1 ? 1 : (P).nq)
+
 // One request: an operator, its right-hand sides and all solver state.
 struct Prob {
     int64_t n;
@@ -94,11 +97,13 @@ struct Prob {
     void* invd;        // [n] VT: 1 / (sigma + sum_s |w_s|), the left scaling (precond == 1)
     RhsState* st;      // [Q]
     void* part;        // [kRedSlots][channels][nchunk][Q] tile partials (Part<MIXED>: F2 or double)
-    unsigned* arrive;  // [kRedSlots]
-    int nchunk, pad;
+    unsigned* arrive;  // [groups][kRedSlots]
+    int nchunk;
+    int nq;            // right-hand sides a block works on: Q, or one group of them (see ReqTable::groups)
     // multigrid right preconditioning (precond == 2); amg == nullptr otherwise
     const AmgHeader* amg;
-    int amg_levels, pad3;
+    int amg_levels;
+    int q0;            // first right-hand side of the group (0: all of them)
     void* ph;                    // [n][Q] VT: M^-1 p
     void* sh;                    // [n][Q] VT: M^-1 s
     float* vy[kAmgMaxLevels];    // per level [n_l][Q]: pre-smoothed y_l = d_l b_l
@@ -232,8 +237,6 @@ __host__ __device__ constexpr int pow2_at_least(int x) { return x <= 1 ? 1 : 2 *
 // (||f|| below about 1.8e19) or the step reports a non-finite residual.
 template <bool MIXED>
 using Part = typename std::conditional<MIXED, F2, double>::type;
-__device__ __forceinline__ F2 part_add(F2 a, F2 b) { return f2_add(a, b); }
-__device__ __forceinline__ double part_add(double a, double b) { return a + b; }
 __device__ __forceinline__ double part_value(F2 a) { return f2_to_double(a); }
 __device__ __forceinline__ double part_value(double a) { return a; }
 template <typename PT>
@@ -268,48 +271,6 @@ __device__ __forceinline__ F2 part_load(const F2* p) {
     return z;
 }
 __device__ __forceinline__ double part_load(const double* p) { return __ldcg(p); }
-
-__device__ __forceinline__ F2 part_shfl_xor(F2 v, int o) {
-    F2 w;
-    w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-    w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-    return w;
-}
-__device__ __forceinline__ double part_shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-
-// Warp totals of E values a lane (E a power of two, at most 32) with a
-// fraction of the shuffles and additions of E separate butterflies.  At each
-// of the first log2 E offsets (16, 8, ...) a lane keeps half of its values --
-// the upper half if its bit at that offset is set -- and adds the partner's
-// copy of them; the remaining offsets add the one value left.  Every value is
-// summed in exactly the pairs and order of a plain xor butterfly over offsets
-// 16, 8, 4, 2, 1 (additions commute), so the totals are those of E separate
-// butterflies, bit for bit.  Returns the total of value `chan` (set here)
-// that this lane ends with; lanes L with L % (32 / E) == 0 hold values
-// 0 .. E-1 once each.
-template <int E, typename PT>
-__device__ __forceinline__ PT warp_sum_multi(PT (&v)[E], int lane, int& chan) {
-    static_assert(E >= 1 && E <= 32 && (E & (E - 1)) == 0, "a power of two, at most 32 values");
-    chan = 0;
-#pragma unroll
-    for (int t = 0; t < 5; t++) {
-        const int o = 16 >> t;
-        const int h = E >> (t + 1);  // values kept after this offset (0: one value left)
-        if (h >= 1) {
-            const bool up = (lane & o) != 0;
-#pragma unroll
-            for (int j = 0; j < (h >= 1 ? h : 1); j++) {
-                const PT send = up ? v[j] : v[j + h];
-                const PT keep = up ? v[j + h] : v[j];
-                v[j] = part_add(keep, part_shfl_xor(send, o));
-            }
-            if (up) chan += h;
-        } else {
-            v[0] = part_add(v[0], part_shfl_xor(v[0], o));
-        }
-    }
-    return v[0];
-}
 
 // A warp's partials of its slice of a tile, channels 0 .. NCH-1 of every
 // right-hand side, into out[ch * QT + q]: in the FP32 flow the F2 products
@@ -349,6 +310,11 @@ __device__ __forceinline__ void tile_partials(const F2 (&af)[NC][QT], const doub
     static_assert(N <= 64, "two groups hold every channel of every right-hand side");
 }
 
+template <typename VT>
+__host__ __device__ constexpr size_t stage_bytes_per_warp(int kmax) {
+    return (size_t)kSlice * kmax * sizeof(int) + (size_t)kSlice * (kmax + 1) * sizeof(VT);
+}
+
 // Per-warp staging of operator slices.  A slice -- 32 rows' k column slots
 // and k+1 weight slots, each 32 consecutive words in the sliced layout, so two
 // contiguous runs -- arrives in the warp's shared memory by two bulk
@@ -357,31 +323,38 @@ __device__ __forceinline__ void tile_partials(const F2 (&af)[NC][QT], const doub
 // before the current one is used, so the operator keeps streaming while the
 // warp gathers and reduces.  The evict-first hint keeps the small, reused
 // Krylov vectors in L2 while the operator streams past.
+// Its state is two registers, kept for the whole launch: what the launch's
+// shape fixes (buffer sizes and addresses, the L2 policy) is formed where it is
+// used, because the steps between the copies are short of registers.
+template <typename VT>
 struct Stager {
-    unsigned char* base;  // this warp's buffers
-    uint32_t bytes;       // one buffer
-    uint32_t val_off;     // where the weights start inside a buffer
-    uint64_t* bar;        // [2] this warp's mbarriers
-    uint64_t pol;
-    uint32_t parity;      // bit b: parity of buffer b's next completion
-    uint32_t busy;        // bit b: a copy into buffer b has not been waited for
-    int nbuf;
-    int next_c;           // tile whose slice was requested ahead (-1: none), in buffer next_b
-    int next_b;
-    bool ok;              // false once a copy missed its wait: nothing more is issued
+    int next_c;    // tile whose slice was requested ahead (-1: none), in buffer next_b
+    uint32_t st;   // bits 0, 1: parity of buffer b's next completion; 2, 3: a copy into buffer b has not
+                   // been waited for; 4: next_b; 5: a copy missed its wait, nothing more is issued
+    static __device__ __forceinline__ uint32_t bytes(int kmax) { return (uint32_t)stage_bytes_per_warp<VT>(kmax); }
+    static __device__ __forceinline__ unsigned char* buffer(int kmax, int nbuf, int b) {
+        extern __shared__ __align__(16) unsigned char stage_smem[];
+        return stage_smem + ((threadIdx.x >> 5) * nbuf + b) * bytes(kmax);
+    }
+    static __device__ __forceinline__ int* col(int kmax, int nbuf, int b) {
+        return reinterpret_cast<int*>(buffer(kmax, nbuf, b));
+    }
+    static __device__ __forceinline__ void* val(int kmax, int nbuf, int b) {
+        return buffer(kmax, nbuf, b) + kSlice * kmax * sizeof(int);
+    }
+    __device__ __forceinline__ bool ok() const { return (st & 32u) == 0; }
 
-    __device__ int* col(int b) const { return reinterpret_cast<int*>(base + b * bytes); }
-    __device__ const void* val(int b) const { return base + b * bytes + val_off; }
-
-    __device__ void issue(int b, const int32_t* colsrc, const void* valsrc, int esize, int k, int64_t slice) {
+    __device__ __forceinline__ void issue(int kmax, int nbuf, uint64_t* bar, int b, const int32_t* colsrc,
+                                          const void* valsrc, int esize, int k, int64_t slice) {
         __syncwarp();  // every lane has consumed what buffer b held
-        if (!ok) return;  // after a missed wait the warp issues nothing more
-        busy |= 1u << b;
+        if (!ok()) return;  // after a missed wait the warp issues nothing more
+        st |= 4u << b;
         if (lane_id() == 0) {
             const uint32_t cb = (uint32_t)(kSlice * k * 4), vb = (uint32_t)(kSlice * (k + 1) * esize);
+            const uint64_t pol = l2_evict_first_policy();
             mbar_expect_tx(&bar[b], cb + vb);
-            bulk_g2s(col(b), colsrc + slice * (int64_t)(kSlice * k), cb, &bar[b], pol);
-            bulk_g2s(base + b * bytes + val_off,
+            bulk_g2s(col(kmax, nbuf, b), colsrc + slice * (int64_t)(kSlice * k), cb, &bar[b], pol);
+            bulk_g2s(val(kmax, nbuf, b),
                      static_cast<const char*>(valsrc) + slice * (int64_t)(kSlice * (k + 1)) * esize, vb, &bar[b],
                      pol);
         }
@@ -389,24 +362,23 @@ struct Stager {
 
     // The buffer holding tile c's slice: requested now unless it was requested
     // ahead; then, with two buffers, requests tile c2's slice ahead (c2 < 0: none).
-    __device__ int acquire(int c, int64_t slice, int c2, int64_t slice2, const int32_t* colsrc, const void* valsrc,
-                           int esize, int k, int* err) {
+    __device__ __forceinline__ int acquire(int kmax, int nbuf, uint64_t* bar, int c, int64_t slice, int c2,
+                                           int64_t slice2, const int32_t* colsrc, const void* valsrc, int esize, int k,
+                                           int* err) {
+        int b = (st >> 4) & 1u;
         if (next_c >= 0 && next_c != c) {  // a slice requested ahead for a tile not taken: let it land first
-            wait(next_b, err);
+            wait(bar, b, err);
             next_c = -1;
         }
-        int b;
-        if (next_c == c) {
-            b = next_b;
-        } else {
-            b = (busy & 1u) ? 1 : 0;
-            issue(b, colsrc, valsrc, esize, k, slice);
+        if (next_c != c) {
+            b = (st & 4u) ? 1 : 0;
+            issue(kmax, nbuf, bar, b, colsrc, valsrc, esize, k, slice);
         }
         next_c = -1;
         if (nbuf == 2 && c2 >= 0) {
-            next_b = b ^ 1;
             next_c = c2;
-            issue(next_b, colsrc, valsrc, esize, k, slice2);
+            st = (st & ~16u) | (b == 0 ? 16u : 0u);
+            issue(kmax, nbuf, bar, b ^ 1, colsrc, valsrc, esize, k, slice2);
         }
         return b;
     }
@@ -414,24 +386,23 @@ struct Stager {
     // Warp-collective bounded wait for buffer b.  A copy that missed its wait
     // stays marked busy with its parity unchanged, so drain() waits for it
     // again before the block's shared memory is released.
-    __device__ bool wait(int b, int* err) {
-        if (!ok) return false;  // nothing was issued since the first miss
-        const bool landed = __all_sync(0xffffffffu, mbar_wait(&bar[b], (parity >> b) & 1u, kStageWaitLimit));
+    __device__ __forceinline__ bool wait(uint64_t* bar, int b, int* err) {
+        if (!ok()) return false;  // nothing was issued since the first miss
+        const bool landed = __all_sync(0xffffffffu, mbar_wait(&bar[b], (st >> b) & 1u, kStageWaitLimit));
         if (landed) {
-            parity ^= 1u << b;
-            busy &= ~(1u << b);
+            st = (st ^ (1u << b)) & ~(4u << b);
         } else {
-            ok = false;
+            st |= 32u;
             if (lane_id() == 0) atomicCAS(err, 0, (int)MVGD_ETIMEOUT);
         }
-        return ok;
+        return ok();
     }
 
     // Before the block's shared memory goes away: bounded waits for every copy
     // still in flight (landed or not, each buffer's wait ends within its limit).
-    __device__ void drain() {
+    __device__ void drain(uint64_t* bar) {
         for (int b = 0; b < 2; b++)
-            if (busy & (1u << b)) mbar_wait(&bar[b], (parity >> b) & 1u, kStageWaitLimit);
+            if (st & (4u << b)) mbar_wait(&bar[b], (st >> b) & 1u, kStageWaitLimit);
     }
 };
 
@@ -580,7 +551,7 @@ __device__ __forceinline__ void restart_row(const Prob& P, int64_t r, int ph, co
         // retry down a different Krylov path ((rh, r) stays positive)
         VT rhv = rr;
         if (S[q].stall > 0) {
-            uint32_t hsh = (uint32_t)e * 2654435761u ^ (uint32_t)S[q].outer * 40503u;
+            uint32_t hsh = (uint32_t)(e + P.q0) * 2654435761u ^ (uint32_t)S[q].outer * 40503u;
             hsh ^= hsh >> 16; hsh *= 0x7feb352du; hsh ^= hsh >> 15; hsh *= 0x846ca68bu; hsh ^= hsh >> 16;
             const double u01 = (double)hsh * (1.0 / 4294967296.0);
             rhv = (VT)(rv * (1.0 + (u01 - 0.5)));
@@ -624,7 +595,7 @@ __device__ __forceinline__ void amg_pre_row(const Prob& P, int64_t r, int ph, co
 #pragma unroll
     for (int q = 0; q < QT; q++) {
         const int64_t e = r * Q + q;
-        if (q >= Q) break;
+        if (q >= MVGD_NQ(P)) break;
         if (ph == P_PRE_A) {
             VT rn = (VT)0;
             if (S[q].pending) {
@@ -677,7 +648,7 @@ __device__ __forceinline__ void amg_pre_rows(const Prob& P, const int64_t (&r)[N
 #pragma unroll
         for (int q = 0; q < QT; q++) {
             a[k][q] = b[k][q] = c[k][q] = w[k][q] = x[k][q] = h1[k][q] = h2[k][q] = (VT)0;
-            if (!ok[k] || q >= Q) continue;
+            if (!ok[k] || q >= MVGD_NQ(P)) continue;
             const int64_t e = r[k] * Q + q;
             if (ph == P_PRE_A && S[q].pending) {
                 a[k][q] = static_cast<const VT*>(P.s)[e];
@@ -699,7 +670,7 @@ __device__ __forceinline__ void amg_pre_rows(const Prob& P, const int64_t (&r)[N
         if (!ok[k]) continue;
 #pragma unroll
         for (int q = 0; q < QT; q++) {
-            if (q >= Q) break;
+            if (q >= MVGD_NQ(P)) break;
             const int64_t e = r[k] * Q + q;
             if (ph == P_PRE_A) {
                 VT rn = a[k][q];
@@ -927,27 +898,37 @@ struct ChunkTable {
     int nchunks, pad;
 };
 
+// A launch of one request may cut its right-hand sides into `groups` of `gq`
+// each: block b then works on group b % groups alone, as block b / groups of
+// gridDim / groups (the grid is a multiple of `groups`).  A right-hand side's
+// arithmetic does not depend on the others of its request, so neither do the
+// results.  Unit counts are a group's.
 struct ReqTable {
     const Prob* const* prob;       // [count]
     ChunkTable fine;               // kCh-row tiles of level 0 (every Krylov phase; V-cycle level 0)
     ChunkTable lvl[kAmgMaxLevels]; // [l], 1 <= l < mlev: kThreads / amg_group(n_l)-row units of level l
-    ChunkTable coarse;             // 8-row groups (a warp each) of every coarsest level
+    ChunkTable coarse;             // groups of coarse_rows rows of every coarsest level
     int mlev;                      // largest (levels - 1) among the requests
     int nreq;                      // requests in the launch (1: every unit is request 0's, no lookups)
+    int groups, gq;                // right-hand-side groups (1 with several requests)
+    int coarse_rows;               // rows of a coarsest-level unit (a warp each, at most 8)
     int G[kAmgMaxLevels];          // [l], l >= 1: amg_group of the launch's rows at level l (see amg_lanes)
 };
+
+// The block's place among those that share its units.
+__device__ __forceinline__ int block_place(const ReqTable& tab) {
+    return tab.groups == 1 ? (int)blockIdx.x : (int)blockIdx.x / tab.groups;
+}
+__device__ __forceinline__ int block_count(const ReqTable& tab) {
+    return tab.groups == 1 ? (int)gridDim.x : (int)gridDim.x / tab.groups;
+}
 
 // Request of unit c of table T, and the unit's place in that request.
 __device__ __forceinline__ int unit_req(const ReqTable& tab, const ChunkTable& T, int c) {
     return tab.nreq == 1 ? 0 : T.chunk_req[c];
 }
-__device__ __forceinline__ int unit_base(const ReqTable& tab, const ChunkTable& T, int ri) {
-    return tab.nreq == 1 ? 0 : T.chunk_base[ri];
-}
-
-template <typename VT>
-__host__ __device__ constexpr size_t stage_bytes_per_warp(int kmax) {
-    return (size_t)kSlice * kmax * sizeof(int) + (size_t)kSlice * (kmax + 1) * sizeof(VT);
+__device__ __forceinline__ int unit_place(const ReqTable& tab, const ChunkTable& T, int ri, int c) {
+    return tab.nreq == 1 ? c : c - T.chunk_base[ri];
 }
 
 // This block has finished `cnt` tiles of request P in a reducing phase: publish
@@ -983,7 +964,7 @@ __device__ __forceinline__ void arrive_and_finalize(const Prob& P, int ph, int s
         constexpr int kPerWarp = (NC * QT + kThreads / 32 - 1) / (kThreads / 32);
         constexpr int kEnt = kPerWarp > 4 ? 4 : kPerWarp;  // entries a warp takes at once
         constexpr int kDeep = kEnt >= 4 ? 2 : 4;  // tiles of an entry in flight a lane
-        const int nchunk = P.nchunk, Q = P.Q, E = nch * Q;
+        const int nchunk = P.nchunk, Q = P.Q, nq = MVGD_NQ(P), E = nch * nq;
         const PT* part = static_cast<const PT*>(P.part) + (int64_t)slot * NC * nchunk * Q;
         for (int e0 = wid; e0 < E; e0 += kEnt * (kThreads / 32)) {  // warp-uniform
             PT acc[kEnt];
@@ -997,7 +978,7 @@ __device__ __forceinline__ void arrive_and_finalize(const Prob& P, int ph, int s
 #pragma unroll
                     for (int d = 0; d < kDeep; d++) {
                         const int l = l0 + 32 * d;
-                        v[u][d] = e < E && l < nchunk ? part_load(part + ((int64_t)(e / Q) * nchunk + l) * Q + e % Q)
+                        v[u][d] = e < E && l < nchunk ? part_load(part + ((int64_t)(e / nq) * nchunk + l) * Q + e % nq)
                                                       : part_zero<PT>();
                     }
                 }
@@ -1012,40 +993,48 @@ __device__ __forceinline__ void arrive_and_finalize(const Prob& P, int ph, int s
                 const int e = e0 + u * (kThreads / 32);
                 if (e >= E) break;  // warp-uniform
                 const PT t = part_warp_sum(acc[u]);
-                if (lane == 0) tot[(e / Q) * QT + e % Q] = part_value(t);
+                if (lane == 0) tot[(e / nq) * QT + e % nq] = part_value(t);
             }
         }
     } else if (*last) {
+        // tiles a batch: a tree over 16 is the sum of two trees over 8, loaded one
+        // after the other (16 doubles of two entries would not fit the registers)
         constexpr int kFinBatch = (QT == 1 && !MIXED) ? 16 : 8;
-        const int nchunk = P.nchunk, Q = P.Q;
-        // two channels (or right-hand sides) at a time: 2 x kFinBatch loads in flight
+        const int nchunk = P.nchunk, Q = P.Q, nq = MVGD_NQ(P);
+        // two channels (or right-hand sides) at a time: 16 loads in flight
 #pragma unroll
         for (int e0 = 0; e0 < NC * QT; e0 += 2) {
             const int e1 = e0 + 1;
-            const bool on0 = e0 / QT < nch && e0 % QT < Q;                   // step-uniform
-            const bool on1 = e1 < NC * QT && e1 / QT < nch && e1 % QT < Q;  // step-uniform
+            const bool on0 = e0 / QT < nch && e0 % QT < nq;                   // step-uniform
+            const bool on1 = e1 < NC * QT && e1 / QT < nch && e1 % QT < nq;  // step-uniform
             PT acc0 = part_zero<PT>(), acc1 = part_zero<PT>();
             if (on0 || on1) {
                 const PT* part = static_cast<const PT*>(P.part);
                 const PT* b0 = &part[((int64_t)slot * NC + e0 / QT) * nchunk * Q + e0 % QT];
                 const PT* b1 = &part[((int64_t)slot * NC + e1 / QT) * nchunk * Q + e1 % QT];
                 for (int l0 = tid; l0 < nchunk; l0 += kThreads * kFinBatch) {
-                    PT v0[kFinBatch], v1[kFinBatch];
+                    PT t0 = part_zero<PT>(), t1 = part_zero<PT>();
+#pragma unroll 1
+                    for (int h = 0; h < kFinBatch; h += 8) {
+                        PT v0[8], v1[8];
 #pragma unroll
-                    for (int u = 0; u < kFinBatch; u++) {
-                        const int l = l0 + u * kThreads;
-                        v0[u] = on0 && l < nchunk ? part_load(b0 + (int64_t)l * Q) : part_zero<PT>();
-                        v1[u] = on1 && l < nchunk ? part_load(b1 + (int64_t)l * Q) : part_zero<PT>();
-                    }
-#pragma unroll
-                    for (int w = 1; w < kFinBatch; w <<= 1)
-#pragma unroll
-                        for (int u = 0; u < kFinBatch; u += 2 * w) {
-                            v0[u] = part_add(v0[u], v0[u + w]);
-                            v1[u] = part_add(v1[u], v1[u + w]);
+                        for (int u = 0; u < 8; u++) {
+                            const int l = l0 + (h + u) * kThreads;
+                            v0[u] = on0 && l < nchunk ? part_load(b0 + (int64_t)l * Q) : part_zero<PT>();
+                            v1[u] = on1 && l < nchunk ? part_load(b1 + (int64_t)l * Q) : part_zero<PT>();
                         }
-                    acc0 = part_add(acc0, v0[0]);
-                    acc1 = part_add(acc1, v1[0]);
+#pragma unroll
+                        for (int w = 1; w < 8; w <<= 1)
+#pragma unroll
+                            for (int u = 0; u < 8; u += 2 * w) {
+                                v0[u] = part_add(v0[u], v0[u + w]);
+                                v1[u] = part_add(v1[u], v1[u + w]);
+                            }
+                        t0 = h == 0 ? v0[0] : part_add(t0, v0[0]);
+                        t1 = h == 0 ? v1[0] : part_add(t1, v1[0]);
+                    }
+                    acc0 = part_add(acc0, t0);
+                    acc1 = part_add(acc1, t1);
                 }
             }
             if (on0) acc0 = part_warp_sum(acc0);
@@ -1066,7 +1055,7 @@ __device__ __forceinline__ void arrive_and_finalize(const Prob& P, int ph, int s
     }
     if (*last) {
         __syncthreads();
-        if (tid < P.Q) {
+        if (tid < MVGD_NQ(P)) {
             RhsState T = S[tid];
             double cv[NC];
 #pragma unroll
@@ -1087,11 +1076,11 @@ enum VStep : int { V_DOWN = 0, V_COARSE = 1, V_UP = 2 };
 // request ri's and this warp's slice of it holds rows (its slice in *slice2);
 // else -1.  Such a tile is staged exactly like tile c, so its slice can be
 // requested ahead.
-__device__ __forceinline__ int next_tile(const ReqTable& tab, const ChunkTable& T, int c, int ri, int64_t nrows,
-                                         int wid, int64_t& slice2) {
-    const int c2 = c + (int)gridDim.x;
+__device__ __forceinline__ int next_tile(const ReqTable& tab, const ChunkTable& T, int c, int nblk, int ri,
+                                         int64_t nrows, int wid, int64_t& slice2) {
+    const int c2 = c + nblk;
     if (c2 >= T.nchunks || unit_req(tab, T, c2) != ri) return -1;
-    slice2 = (int64_t)(c2 - unit_base(tab, T, ri)) * (kCh / kSlice) + wid;
+    slice2 = (int64_t)unit_place(tab, T, ri, c2) * (kCh / kSlice) + wid;
     return slice2 * kSlice < nrows ? c2 : -1;
 }
 
@@ -1099,7 +1088,6 @@ template <bool MIXED, int QT, bool AMG>
 __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     k_solve(ReqTable tab, Ctl ctl, int iter_budget, int kmax, int nbuf) {
     using VT = typename std::conditional<MIXED, float, double>::type;
-    extern __shared__ __align__(16) unsigned char stage_smem[];
     __shared__ RhsState S[QT];
     __shared__ __align__(16) Prob sP;
     __shared__ __align__(16) AmgHeader sH;
@@ -1118,24 +1106,16 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     __shared__ float vagg[kThreads / kAmgAgg];  // a block's row residuals on a small level (agg_sum)
     __shared__ __align__(8) uint64_t stage_bar[kThreads / 32][2];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int bid = block_place(tab), nblk = block_count(tab);
     // this warp's nbuf slice buffers: kmax column slots, then kmax + 1 weight slots each
-    Stager st;
-    st.bytes = (uint32_t)stage_bytes_per_warp<VT>(kmax);
-    st.val_off = (uint32_t)(kSlice * kmax * sizeof(int));
-    st.base = stage_smem + (size_t)wid * nbuf * st.bytes;
-    st.bar = stage_bar[wid];
-    st.pol = 0;
-    st.parity = 0;
-    st.busy = 0;
-    st.nbuf = nbuf;
+    Stager<VT> st;
     st.next_c = -1;
-    st.next_b = 0;
-    st.ok = true;
+    st.st = 0;
+#define MVGD_STAGE_BAR stage_bar[threadIdx.x >> 5]
     if (lane == 0) {
-        mbar_init(&st.bar[0], 1);
-        mbar_init(&st.bar[1], 1);
+        mbar_init(&stage_bar[wid][0], 1);
+        mbar_init(&stage_bar[wid][1], 1);
         fence_mbar_init();
-        st.pol = l2_evict_first_policy();
     }
     __syncthreads();
 
@@ -1155,7 +1135,8 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     auto load_desc = [&](int ri) {
         if (ri == desc) return;
         __syncthreads();  // every thread is done with the previous one
-        const unsigned long long* gp = reinterpret_cast<const unsigned long long*>(tab.prob[ri]);
+        const unsigned long long* gp =
+            reinterpret_cast<const unsigned long long*>(tab.prob[ri]);
         for (int w = tid; w < (int)(sizeof(Prob) / 8); w += kThreads)
             reinterpret_cast<unsigned long long*>(&sP)[w] = __ldcg(gp + w);
         __syncthreads();
@@ -1165,6 +1146,25 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
                 reinterpret_cast<unsigned long long*>(&sH)[w] = __ldcg(gh + w);
             __syncthreads();
             if (tid == 0) sP.amg = &sH;
+            __syncthreads();
+        }
+        if (tab.groups > 1) {  // this group's columns of every [n][Q] array, its states, partials and counters
+            if (tid == 0) {
+                const int g = (int)blockIdx.x % tab.groups, q0 = g * tab.gq;
+                auto shift = [&](auto*& p) { if (p) p += q0; };
+                auto shift_vt = [&](void*& p) { if (p) p = static_cast<VT*>(p) + q0; };
+                shift(sP.f); shift(sP.u); shift(sP.r64); shift(sP.st);
+                shift_vt(sP.x); shift_vt(sP.xb); shift_vt(sP.r); shift_vt(sP.rh);
+                shift_vt(sP.p[0]); shift_vt(sP.p[1]); shift_vt(sP.v[0]); shift_vt(sP.v[1]);
+                shift_vt(sP.s); shift_vt(sP.t); shift_vt(sP.ph); shift_vt(sP.sh);
+                for (int l = 0; l < kAmgMaxLevels; l++) {
+                    shift(sP.vy[l]); shift(sP.vr[l]); shift(sP.vb[l]); shift(sP.vx[l]);
+                }
+                sP.part = static_cast<Part<MIXED>*>(sP.part) + q0;
+                sP.arrive += g * kRedSlots;
+                sP.nq = tab.gq;
+                sP.q0 = q0;
+            }
             __syncthreads();
         }
         desc = ri;
@@ -1182,7 +1182,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
         if (AMG && fits) fits = P.amg->n == P.n && P.amg->k == P.k;
         if (!fits && tid == 0) atomicCAS(ctl.err, 0, (int)MVGD_EINVAL);
         if (tid < QT) {
-            if (tid < P.Q && fits) {
+            if (tid < MVGD_NQ(P) && fits) {
                 load_state(S[tid], P.st + tid);
             } else {  // a slot past the request's RHS count: no work of any kind
                 S[tid].mode = M_DONE;
@@ -1225,15 +1225,15 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
                 const Part<MIXED> v = part_add(part_add(part_add(rw[0], rw[W]), part_add(rw[2 * W], rw[3 * W])),
                                                part_add(part_add(rw[4 * W], rw[5 * W]), part_add(rw[6 * W], rw[7 * W])));
                 const int ch = j / QT, q = j % QT;
-                if (q < P.Q)
+                if (q < MVGD_NQ(P))
                     static_cast<Part<MIXED>*>(P.part)[(((int64_t)slot * NC + ch) * P.nchunk + red_lc[t]) * P.Q + q] = v;
             }
             __syncthreads();
             nred = 0;
         };
-        for (int c = blockIdx.x;; c += gridDim.x) {
+        for (int c = bid;; c += nblk) {
             const int ri = c < tab.fine.nchunks ? unit_req(tab, tab.fine, c) : -1;
-            if (ri != cur) {
+            if (ri != cur || ri < 0) {  // (a block may have no level-0 tile at all)
                 // leaving request `cur`: publish this block's tiles of it
                 if (cur >= 0 && reduce && tiles > 0) {
                     flush(sP);  // still request cur's descriptor
@@ -1246,7 +1246,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
             }
             if (all_done) continue;  // the whole request is finished: no work, no arrival
             const Prob& P = sP;
-            const int lc = c - unit_base(tab, tab.fine, ri);
+            const int lc = unit_place(tab, tab.fine, ri, c);
             const int64_t r = (int64_t)lc * kCh + tid;
             const int64_t slice = (int64_t)lc * (kCh / kSlice) + wid;
             F2 af[NC][QT];
@@ -1256,17 +1256,17 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
 #pragma unroll
                 for (int q = 0; q < QT; q++) { af[ch][q].hi = 0.0f; af[ch][q].lo = 0.0f; ad[ch][q] = 0.0; }
             // warp-uniform: lane 0 stages the whole slice and every lane waits for it
-            const bool staged = (ph == P_A || ph == P_B) && any_inner && slice * kSlice < P.n && st.ok;
+            const bool staged = (ph == P_A || ph == P_B) && any_inner && slice * kSlice < P.n && st.ok();
             if (staged) {
                 int64_t slice2 = 0;
-                const int cn = next_tile(tab, tab.fine, c, ri, P.n, wid, slice2);
+                const int cn = next_tile(tab, tab.fine, c, nblk, ri, P.n, wid, slice2);
                 // FP32 multigrid flow: the hierarchy's level-0 weights (the operator's hi
                 // values, copied at set-up), the array the V-cycle's level-0 steps read too
                 const void* vsrc = (AMG && MIXED) ? static_cast<const void*>(P.amg->lv[0].val) : P.val;
-                const int b = st.acquire(c, slice, cn, slice2, P.col, vsrc, (int)sizeof(VT), P.k, ctl.err);
-                const int* colS = st.col(b);
-                const VT* valS = static_cast<const VT*>(st.val(b));
-                auto landed = [&]() { return st.wait(b, ctl.err); };
+                const int b = st.acquire(kmax, nbuf, MVGD_STAGE_BAR, c, slice, cn, slice2, P.col, vsrc, (int)sizeof(VT), P.k, ctl.err);
+                const int* colS = st.col(kmax, nbuf, b);
+                const VT* valS = static_cast<const VT*>(st.val(kmax, nbuf, b));
+                auto landed = [&]() { return st.wait(MVGD_STAGE_BAR, b, ctl.err); };
                 if constexpr (AMG) amg_spmv_row<MIXED, QT>(P, r, r < P.n, ph, S, inner, af, ad, colS, valS, landed);
                 else spmv_row<MIXED, QT>(P, r, r < P.n, ph, S, inner, c1, c2, af, ad, colS, valS, landed);
             }
@@ -1323,18 +1323,17 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     // x into u).  The rows and their arithmetic are those of fine_phase.
     auto pre_phase = [&](int ph) -> bool {
         constexpr int NT = MIXED ? (QT == 1 ? 4 : 2) : (QT == 1 ? 2 : 1);  // operands in registers
-        const int G = (int)gridDim.x;
-        for (int c = blockIdx.x; c < tab.fine.nchunks;) {
+        const int G = nblk;
+        for (int c = bid; c < tab.fine.nchunks;) {
             const int ri = unit_req(tab, tab.fine, c);
             if (ri != held) enter(ri, ph);
             int n = 1;
             while (n < NT && c + n * G < tab.fine.nchunks && unit_req(tab, tab.fine, c + n * G) == ri) n++;
             if (!all_done) {
                 const Prob& P = sP;
-                const int base = unit_base(tab, tab.fine, ri);
                 if (any_restart) {
                     for (int k = 0; k < n; k++) {
-                        const int64_t r = (int64_t)(c + k * G - base) * kCh + tid;
+                        const int64_t r = (int64_t)unit_place(tab, tab.fine, ri, c + k * G) * kCh + tid;
                         if (r < P.n) amg_pre_row<MIXED, QT>(P, r, ph, S, inner, restart);
                     }
                 } else {
@@ -1342,7 +1341,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
                     bool ok[NT];
 #pragma unroll
                     for (int k = 0; k < NT; k++) {
-                        rows[k] = (int64_t)(c + k * G - base) * kCh + tid;
+                        rows[k] = (int64_t)unit_place(tab, tab.fine, ri, c + k * G) * kCh + tid;
                         ok[k] = k < n && rows[k] < P.n;
                     }
                     amg_pre_rows<MIXED, QT, NT>(P, rows, ok, ph, S, inner);
@@ -1361,7 +1360,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     auto vstep = [&](int kind, int l, int side) -> bool {
         const ChunkTable& T = kind == V_COARSE ? tab.coarse : (l == 0 ? tab.fine : tab.lvl[l]);
         int cur = -1;
-        for (int c = blockIdx.x; c < T.nchunks; c += gridDim.x) {
+        for (int c = bid; c < T.nchunks; c += nblk) {
             const int ri = unit_req(tab, T, c);
             if (ri != cur) {
                 cur = ri;
@@ -1374,23 +1373,20 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
             if (!any_inner || (kind != V_COARSE && l >= m)) continue;
             const AmgHeader& H = *P.amg;
             const int Q = P.Q;
-            const int lc = c - unit_base(tab, T, ri);
+            const int lc = unit_place(tab, T, ri, c);
             const VT* B0 = static_cast<const VT*>(side == 0 ? P.p[0] : P.s);
             VT* X0 = static_cast<VT*>(side == 0 ? P.ph : P.sh);
             if (kind == V_COARSE) {
-                const int64_t rho = (int64_t)lc * (kThreads / kWarp) + wid;  // a warp per row
-                if (rho >= H.nc) continue;
-#pragma unroll
-                for (int q = 0; q < QT; q++) {
-                    if (!inner[q]) continue;
-                    float x;
-                    if (m == 0) x = coarse_row(H, rho, [&](int64_t cc) { return (float)B0[cc * Q + q]; });
-                    else x = coarse_row(H, rho, [&](int64_t cc) { return P.vb[m][cc * Q + q]; });
-                    if (lane == 0) {
-                        if (m == 0) X0[rho * Q + q] = (VT)x;
-                        else P.vx[m][rho * Q + q] = x;
-                    }
-                }
+                // a warp per row, every right-hand side at once
+                const int64_t rho = (int64_t)lc * tab.coarse_rows + wid;
+                if (wid >= tab.coarse_rows || rho >= H.nc) continue;
+                auto store = [&](int q, float x) {
+                    if (q >= MVGD_NQ(P) || S[q].mode != M_INNER) return;
+                    if (m == 0) X0[rho * Q + q] = (VT)x;
+                    else P.vx[m][rho * Q + q] = x;
+                };
+                if (m == 0) coarse_rows<QT>(H, rho, B0, Q, store);
+                else coarse_rows<QT>(H, rho, P.vb[m], Q, store);
                 continue;
             }
             const int64_t nl = H.lv[l].n;
@@ -1407,13 +1403,13 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
             const float* w0S = nullptr;
             int b = 0;
             if (l == 0) {
-                if (!st.ok) continue;
+                if (!st.ok()) continue;
                 const int64_t slice = (int64_t)lc * (kCh / kSlice) + wid;
                 int64_t slice2 = 0;
-                const int cn = next_tile(tab, tab.fine, c, ri, nl, wid, slice2);
-                b = st.acquire(c, slice, cn, slice2, P.col, H.lv[0].val, 4, P.k, ctl.err);
-                colS = st.col(b);
-                w0S = static_cast<const float*>(st.val(b));
+                const int cn = next_tile(tab, tab.fine, c, nblk, ri, nl, wid, slice2);
+                b = st.acquire(kmax, nbuf, MVGD_STAGE_BAR, c, slice, cn, slice2, P.col, H.lv[0].val, 4, P.k, ctl.err);
+                colS = st.col(kmax, nbuf, b);
+                w0S = static_cast<const float*>(st.val(kmax, nbuf, b));
             }
             const float sig = (float)P.sigma;
             const int k = P.k;
@@ -1431,7 +1427,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
                 }
                 if (l == 0) {
                     // level 0: every right-hand side in one pass over the neighbours
-                    if (!st.wait(b, ctl.err)) continue;
+                    if (!st.wait(MVGD_STAGE_BAR, b, ctl.err)) continue;
                     float ay[QT];
 #pragma unroll
                     for (int q = 0; q < QT; q++) ay[q] = 0.0f;
@@ -1462,7 +1458,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
                 }
                 if (l == 0) {
                     // level 0: x = y + x_c + d (r - A_0 P x_c), every right-hand side in one pass
-                    if (!st.wait(b, ctl.err) || !valid) continue;
+                    if (!st.wait(MVGD_STAGE_BAR, b, ctl.err) || !valid) continue;
                     float xc[QT], apx[QT];
                     load_row<QT>(Xc, r / kAmgAgg, Q, xc);
                     a0_rows_staged<QT>(colS, w0S, lane, k, sig, xc, apx,
@@ -1525,7 +1521,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     }
     // copies still landing (a missed wait): bounded waits before the block's
     // shared memory is released
-    st.drain();
+    st.drain(MVGD_STAGE_BAR);
 }
 
 // ------------------------------------------------------------------------------
@@ -1559,7 +1555,7 @@ ReqLayout req_layout(void* ws, int64_t n, int Q, int prec, int precond) {
     L.prob = cv.take<Prob>(1);
     L.st = cv.take<RhsState>(Q);
     L.part = cv.take<double>(kRedSlots * chan_count(precond == 2) * nchunk * Q);
-    L.arrive = cv.take<unsigned>(kRedSlots);
+    L.arrive = cv.take<unsigned>(kRedSlots * 8);  // a set for each right-hand-side group (256 bytes either way)
     L.info = cv.take<mvgd_solve_info>(Q);
     L.fs = cv.take<double>(n * Q);
     L.us = cv.take<double>(n * Q);
@@ -1640,7 +1636,7 @@ __global__ void k_request_init(Prob P, Prob* dst, int64_t n) {
         T.best_flag = T.fold_best = T.since_best = T.pending = 0;
         P.st[threadIdx.x] = T;
     }
-    if (blockIdx.x == 0 && threadIdx.x < kRedSlots) P.arrive[threadIdx.x] = 0;
+    if (blockIdx.x == 0 && threadIdx.x < kRedSlots * 8) P.arrive[threadIdx.x] = 0;
 }
 
 // Left scaling of the Krylov system: d_r = sigma + sum_s |w_rs| over the row's
@@ -1734,6 +1730,25 @@ __global__ void k_build_table(TableArgs A, int base, const Prob** prob, int* chu
     }
 }
 
+// The tables, control words and counts of a launch of one request: it needs no
+// unit tables (see unit_req).
+__global__ void k_start_one(const Prob* req, const Prob** prob, unsigned* bar, int* words) {
+    if (threadIdx.x != 0) return;
+    prob[0] = req;
+    bar[0] = 0;
+    bar[1] = 0;
+    int act = 0, rst = 0;
+    for (int q = 0; q < req->Q; q++) {
+        const int md = __ldcg(&req->st[q].mode);
+        act += md != M_DONE;
+        rst += md == M_RESTART;
+    }
+    words[0] = 0;  // err
+    words[1] = act;
+    words[2] = rst;
+    words[3] = 0;  // stop
+}
+
 // Counts running and restarting right-hand sides of the listed requests.
 __global__ void k_count_active(const Prob** prob, int count, int* words) {
     __shared__ int act, rst;
@@ -1788,25 +1803,46 @@ int stage_buffers(int kmax) {
     return 1;
 }
 
+// Resident blocks of one instantiation (0: a CUDA error).
+template <bool MIXED, int QT, bool AMG>
+int solve_capacity(int kmax, size_t* smem_out = nullptr) {
+    using VT = typename std::conditional<MIXED, float, double>::type;
+    auto fn = k_solve<MIXED, QT, AMG>;
+    const size_t smem = stage_bytes_per_warp<VT>(kmax) * (kThreads / kWarp) * stage_buffers<VT>(kmax);
+    int dev = 0, sms = 0, per_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem) != cudaSuccess)
+        return 0;
+    const int want = tuned_solver_blocks_per_sm();
+    if (want > 0 && want < per_sm) per_sm = want;
+    if (smem_out) *smem_out = smem;
+    return sms * per_sm;
+}
+
 template <bool MIXED, int QT, bool AMG>
 mvgd_status launch_solve(const ReqTable& tab, Ctl ctl, int budget, int kmax, cudaStream_t s) {
     using VT = typename std::conditional<MIXED, float, double>::type;
-    auto fn = k_solve<MIXED, QT, AMG>;
+    size_t smem = 0;
+    int grid = solve_capacity<MIXED, QT, AMG>(kmax, &smem);
+    if (grid < 1) return MVGD_ECUDA;
+    // a block for every unit of the step that has most of them (a level whose rows
+    // must take many lanes, or the coarsest one of a small system, can have more
+    // units than level 0)
+    int units = tab.fine.nchunks;
+    if (AMG) {
+        for (int l = 1; l < tab.mlev; l++) units = units > tab.lvl[l].nchunks ? units : tab.lvl[l].nchunks;
+        units = units > tab.coarse.nchunks ? units : tab.coarse.nchunks;
+    }
+    units *= tab.groups;
+    if (grid > units) grid = units;
+    grid -= grid % tab.groups;  // units is a multiple of groups, and groups <= 8 blocks always fit
     int nbuf = stage_buffers<VT>(kmax);
-    const size_t smem = stage_bytes_per_warp<VT>(kmax) * (kThreads / kWarp) * nbuf;
-    int dev = 0, sms = 0, per_sm = 0;
-    MVGD_CUDA_TRY(cudaGetDevice(&dev));
-    MVGD_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    MVGD_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    MVGD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem));
-    if (per_sm < 1) return MVGD_ECUDA;
-    const int want = tuned_solver_blocks_per_sm();
-    if (want > 0 && want < per_sm) per_sm = want;
-    int grid = sms * per_sm;
-    if (grid > tab.fine.nchunks) grid = tab.fine.nchunks;
     ReqTable t = tab;
     void* args[] = {(void*)&t, (void*)&ctl, (void*)&budget, (void*)&kmax, (void*)&nbuf};
-    MVGD_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)fn, dim3(grid), dim3(kThreads), args, smem, s));
+    MVGD_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_solve<MIXED, QT, AMG>, dim3(grid), dim3(kThreads), args,
+                                              smem, s));
     return MVGD_OK;
 }
 
@@ -1816,6 +1852,28 @@ mvgd_status dispatch_q(int Q, const ReqTable& tab, Ctl ctl, int budget, int kmax
     if (Q <= 2) return launch_solve<MIXED, 2, AMG>(tab, ctl, budget, kmax, s);
     if (Q <= 4) return launch_solve<MIXED, 4, AMG>(tab, ctl, budget, kmax, s);
     return launch_solve<MIXED, 8, AMG>(tab, ctl, budget, kmax, s);
+}
+
+// Right-hand sides a group of a one-request launch takes (Q: no split): the
+// fewest (1, 2 or 4, dividing Q) whose level-0 units all fit the GPU at once.
+// A small system with several right-hand sides leaves most SMs idle, and its
+// steps last as long as one SM needs for all of them -- in FP64 above all,
+// where an SM's pipe takes 2 FMAs a clock.  Once a second round of units would
+// start, the operator read again for each group costs more than it gives.
+// 16,000 rows x 8 right-hand sides in FP64: 257 us an iteration unsplit, 115 in
+// groups of two; 7,001 rows x 4 in FP32: 124 and 64.
+template <bool MIXED, bool AMG>
+int rhs_group(int Q, int tiles, int kmax) {
+    const int64_t t = tiles;
+    if (t * Q <= solve_capacity<MIXED, 1, AMG>(kmax)) return 1;
+    if (Q > 2 && Q % 2 == 0 && t * (Q / 2) <= solve_capacity<MIXED, 2, AMG>(kmax)) return 2;
+    if (Q > 4 && Q % 4 == 0 && t * (Q / 4) <= solve_capacity<MIXED, 4, AMG>(kmax)) return 4;
+    return Q;
+}
+
+int rhs_group(bool mixed, bool amg, int Q, int tiles, int kmax) {
+    if (mixed) return amg ? rhs_group<true, true>(Q, tiles, kmax) : rhs_group<true, false>(Q, tiles, kmax);
+    return amg ? rhs_group<false, true>(Q, tiles, kmax) : rhs_group<false, false>(Q, tiles, kmax);
 }
 
 int gather_blocks(int64_t elems) {
@@ -1891,7 +1949,7 @@ MVGD_API mvgd_status mvgd_request_init(void* req_ws, size_t req_bytes, const mvg
     P.part = W.part;
     P.arrive = W.arrive;
     P.nchunk = (int)((n + kCh - 1) / kCh);
-    P.pad = 0;
+    P.nq = nrhs;
     P.rtol = opts->rtol;
     P.inner_rtol = mixed ? opts->inner_rtol : 0.0;
     P.maxit = opts->maxit;
@@ -1900,7 +1958,7 @@ MVGD_API mvgd_status mvgd_request_init(void* req_ws, size_t req_bytes, const mvg
     P.pad2 = 0;
     P.amg = opts->precond == 2 ? static_cast<const AmgHeader*>(opts->amg) : nullptr;
     P.amg_levels = W.nlev;
-    P.pad3 = 0;
+    P.q0 = 0;
     P.ph = W.vec[10];
     P.sh = W.vec[11];
     for (int l = 0; l < kAmgMaxLevels; l++) {
@@ -1952,17 +2010,44 @@ MVGD_API mvgd_status mvgd_iterate(const mvgd_request* reqs, int32_t count, int32
     tab.prob = C.prob;
     tab.mlev = mlev;
     tab.nreq = count;
-    const int qt = maxQ <= 1 ? 1 : (maxQ <= 2 ? 2 : (maxQ <= 4 ? 4 : 8));  // the solver's right-hand-side width
+    const bool mixed = prec == MVGD_FP32_REFINE;
+    // one request: its right-hand sides in groups where they leave SMs idle
+    const int gq = count == 1 && maxQ > 1
+                       ? rhs_group(mixed, amg, maxQ, (int)((reqs[0].n + kCh - 1) / kCh), kmax) : maxQ;
+    tab.groups = maxQ / gq;
+    tab.gq = gq;
+    const int qt = gq <= 1 ? 1 : (gq <= 2 ? 2 : (gq <= 4 ? 4 : 8));  // the solver's right-hand-side width
+    // lanes of a coarse level's rows: what fills the blocks that level 0 brings
+    // along, and no more.  A small system's levels could use more blocks, but every
+    // grid barrier then waits for those too: 20,000 rows have 79 tiles; with 313
+    // blocks (32 lanes a row on level 1) each of the 14 steps of an iteration took
+    // 0.7 to 1 us longer than with 79 blocks and 8 lanes a row.
+    int64_t threads = 0;
+    for (int i = 0; i < count; i++) threads += ((reqs[i].n + kCh - 1) / kCh) * kThreads;
+    threads *= tab.groups;
     for (int l = 0; l < kAmgMaxLevels; l++) {
         int64_t rows = 0;
         for (int i = 0; amg && l > 0 && i < count; i++) {
             int64_t sizes[kAmgMaxLevels];
             const int nl = amg_levels(reqs[i].n, sizes);
-            if (l < nl - 1) rows += sizes[l];
+            if (l < nl - 1) rows += sizes[l] * tab.groups;
         }
-        tab.G[l] = l == 0 || rows == 0 ? 1 : amg_group(rows);
+        int g = l == 0 || rows == 0 ? 1 : amg_group(rows);
+        while (g > 1 && rows * g > threads) g >>= 1;
+        tab.G[l] = g;
     }
-    // table t: 0 = level-0 tiles, 1 .. mlev-1 = level-t tiles, kAmgMaxLevels = coarsest rows by 8
+    // rows of the coarsest level a block takes: eight (a warp each), fewer while the
+    // blocks of one request last -- the FP64 sums of eight warps queue for one SM's pipe
+    tab.coarse_rows = kThreads / kWarp;
+    if (count == 1 && amg) {
+        int64_t sizes[kAmgMaxLevels];
+        const int64_t nc = sizes[amg_levels(reqs[0].n, sizes) - 1];
+        const int64_t blocks = threads / tab.groups / kThreads < kAmgLanesOnePass / kThreads / tab.groups
+                                   ? threads / tab.groups / kThreads : kAmgLanesOnePass / kThreads / tab.groups;
+        while (tab.coarse_rows > 1 && (nc + tab.coarse_rows / 2 - 1) / (tab.coarse_rows / 2) <= blocks)
+            tab.coarse_rows /= 2;
+    }
+    // table t: 0 = level-0 tiles, 1 .. mlev-1 = level-t tiles, kAmgMaxLevels = coarsest rows
     for (int t = 0; t <= kAmgMaxLevels; t++) {
         const bool coarse = t == kAmgMaxLevels;
         if (t > 0 && (!amg || (!coarse && t >= mlev))) continue;
@@ -1977,7 +2062,7 @@ MVGD_API mvgd_status mvgd_iterate(const mvgd_request* reqs, int32_t count, int32
                 int64_t sizes[kAmgMaxLevels];
                 const int nl = amg ? amg_levels(R.n, sizes) : 1;
                 if (t == 0) A.nchunk[i] = (int)((R.n + kCh - 1) / kCh);
-                else if (coarse) A.nchunk[i] = (int)((sizes[nl - 1] + kThreads / kWarp - 1) / (kThreads / kWarp));
+                else if (coarse) A.nchunk[i] = (int)((sizes[nl - 1] + tab.coarse_rows - 1) / tab.coarse_rows);
                 else if (t < nl - 1) {
                     const int64_t rows = kThreads / amg_lanes(tab.G[t], sizes[t], qt);  // rows per unit
                     A.nchunk[i] = (int)((sizes[t] + rows - 1) / rows);
@@ -1986,15 +2071,20 @@ MVGD_API mvgd_status mvgd_iterate(const mvgd_request* reqs, int32_t count, int32
                 }
                 units += A.nchunk[i];
             }
-            k_build_table<<<1, 256, 0, s>>>(A, g, t == 0 ? C.prob : nullptr, C.chunk_req[t], C.chunk_base[t], C.bar,
-                                            C.words, t == 0 && g == 0);
+            if (count > 1)
+                k_build_table<<<1, 256, 0, s>>>(A, g, t == 0 ? C.prob : nullptr, C.chunk_req[t], C.chunk_base[t],
+                                                C.bar, C.words, t == 0 && g == 0);
         }
         ChunkTable& T = coarse ? tab.coarse : (t == 0 ? tab.fine : tab.lvl[t]);
         T.chunk_req = C.chunk_req[t];
         T.chunk_base = C.chunk_base[t];
         T.nchunks = units;
     }
-    k_count_active<<<1, 256, 0, s>>>(C.prob, count, C.words);
+    if (count > 1) {
+        k_count_active<<<1, 256, 0, s>>>(C.prob, count, C.words);
+    } else {
+        k_start_one<<<1, 32, 0, s>>>(reinterpret_cast<const Prob*>(reqs[0].workspace), C.prob, C.bar, C.words);
+    }
     Ctl ctl;
     ctl.bar.count = C.bar;
     ctl.bar.gen = C.bar + 1;
@@ -2007,12 +2097,12 @@ MVGD_API mvgd_status mvgd_iterate(const mvgd_request* reqs, int32_t count, int32
     ctl.trace = g_trace_on;
     ctl.withhold = take_withhold() ? 1 : 0;
     mvgd_status st;
-    if (prec == MVGD_FP32_REFINE)
-        st = amg ? dispatch_q<true, true>(maxQ, tab, ctl, max_iterations, kmax, s)
-                 : dispatch_q<true, false>(maxQ, tab, ctl, max_iterations, kmax, s);
+    if (mixed)
+        st = amg ? dispatch_q<true, true>(gq, tab, ctl, max_iterations, kmax, s)
+                 : dispatch_q<true, false>(gq, tab, ctl, max_iterations, kmax, s);
     else
-        st = amg ? dispatch_q<false, true>(maxQ, tab, ctl, max_iterations, kmax, s)
-                 : dispatch_q<false, false>(maxQ, tab, ctl, max_iterations, kmax, s);
+        st = amg ? dispatch_q<false, true>(gq, tab, ctl, max_iterations, kmax, s)
+                 : dispatch_q<false, false>(gq, tab, ctl, max_iterations, kmax, s);
     if (st != MVGD_OK) return st;
     k_mark_exit<<<1, 256, 0, s>>>(C.prob, count, C.words);
     return launch_status();

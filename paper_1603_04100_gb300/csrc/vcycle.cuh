@@ -53,24 +53,25 @@ __device__ __forceinline__ float a0_row_staged(const int* colS, const float* w, 
     return sigma * xi - acc;
 }
 
-// Row j of an [n][Q] array into x[0..QT) (zeros past Q).  When Q == QT is 2,
-// 4 or 8 the row is one or two aligned vector loads (workspace arrays start on
-// 256 bytes), else Q scalar loads: a gather of all right-hand sides at a
-// neighbour costs one memory instruction instead of Q.
+// Row j of an [n][Q] array into x[0..QT) (zeros past Q).  When QT is 2, 4 or 8
+// and divides Q the row is one or two aligned vector loads (workspace arrays
+// start on 256 bytes, a group of QT columns on its own size), else scalar
+// loads: a gather of all right-hand sides at a neighbour costs one memory
+// instruction instead of QT.
 template <int QT, typename T>
 __device__ __forceinline__ void load_row(const T* X, int64_t j, int Q, T (&x)[QT]) {
     if constexpr (QT == 2 && sizeof(T) == 4) {
-        if (Q == 2) {
-            const float2 v = reinterpret_cast<const float2*>(X)[j];
+        if (Q % 2 == 0) {
+            const float2 v = *reinterpret_cast<const float2*>(X + j * Q);
             x[0] = v.x;
             x[1] = v.y;
             return;
         }
     } else if constexpr ((QT == 4 || QT == 8) && sizeof(T) == 4) {
-        if (Q == QT) {
+        if (Q % QT == 0) {
 #pragma unroll
             for (int h = 0; h < QT / 4; h++) {
-                const float4 v = reinterpret_cast<const float4*>(X)[j * (QT / 4) + h];
+                const float4 v = reinterpret_cast<const float4*>(X + j * Q)[h];
                 x[4 * h] = v.x;
                 x[4 * h + 1] = v.y;
                 x[4 * h + 2] = v.z;
@@ -79,10 +80,10 @@ __device__ __forceinline__ void load_row(const T* X, int64_t j, int Q, T (&x)[QT
             return;
         }
     } else if constexpr (QT >= 2 && QT <= 8 && (QT & (QT - 1)) == 0 && sizeof(T) == 8) {
-        if (Q == QT) {
+        if (Q % QT == 0) {
 #pragma unroll
             for (int h = 0; h < QT / 2; h++) {
-                const double2 v = reinterpret_cast<const double2*>(X)[j * (QT / 2) + h];
+                const double2 v = reinterpret_cast<const double2*>(X + j * Q)[h];
                 x[2 * h] = v.x;
                 x[2 * h + 1] = v.y;
             }
@@ -141,18 +142,35 @@ __device__ __forceinline__ void al_rows_m(const AmgLevel& Lv, int64_t r, bool va
         // the slice's widest row, rounded up to whole groups of V slots: every row
         // is padded with (own row, 0) to the full stride, whose terms add exact zeros
         const int w = (Lv.sw[r / kSlice] + V - 1) & ~(V - 1);
-        constexpr int kUnroll = M >= 4 ? 1 : 4 / M;  // about four slots in flight a lane
-#pragma unroll kUnroll
-        for (int s0 = 0; s0 < w; s0 += V) {
+        // eight slots in flight a lane with one right-hand side (four with more), every
+        // load issued before the first use: a level of 131,072 rows has a lane a row,
+        // and its step is a chain of as many column -> x round trips to L2 as batches.
+        // Left to the compiler to unroll, four at a time, the level-1 steps of 1M
+        // points took 19 and 13 us (down, up); 16.4 and 12.5 with four as written
+        // here, 13.4 and 11.9 with eight
+        constexpr int kBatch = QT == 1 ? (M >= 8 ? 1 : 8 / M) : (M >= 4 ? 1 : 4 / M);
+        for (int s0 = 0; s0 < w; s0 += V * kBatch) {
+            float a[kBatch][M], x[kBatch][M][QT];
+            int32_t c[kBatch][M];
 #pragma unroll
-            for (int m = 0; m < M; m++) {
-                const int64_t e = base + (int64_t)(s0 + j + m * G) * kSlice;
-                const float a = Lv.val[e];
-                float x[QT];
-                xrow((int64_t)Lv.col[e], x);  // every right-hand side of the neighbour at once
+            for (int b = 0; b < kBatch; b++)
 #pragma unroll
-                for (int q = 0; q < QT; q++) acc[m][q] = fmaf(a, x[q] - xi[q], acc[m][q]);
-            }
+                for (int m = 0; m < M; m++) {
+                    const int64_t e = base + (int64_t)(s0 + b * V + j + m * G) * kSlice;
+                    const bool on = b == 0 || s0 + b * V < w;  // past the row: (own row, 0), an exact zero
+                    c[b][m] = on ? Lv.col[e] : (int32_t)r;
+                    a[b][m] = on ? Lv.val[e] : 0.0f;
+                }
+#pragma unroll
+            for (int b = 0; b < kBatch; b++)
+#pragma unroll
+                for (int m = 0; m < M; m++) xrow((int64_t)c[b][m], x[b][m]);
+#pragma unroll
+            for (int b = 0; b < kBatch; b++)
+#pragma unroll
+                for (int m = 0; m < M; m++)
+#pragma unroll
+                    for (int q = 0; q < QT; q++) acc[m][q] = fmaf(a[b][m], x[b][m][q] - xi[q], acc[m][q]);
         }
     }
     for (int o = 1; o < G; o <<= 1)
@@ -272,13 +290,47 @@ __device__ __forceinline__ float vup_row(const AmgHeader& H, int l, int G, int64
 // FP32 product with the inverse carries cond(A_c) ~ 1e4 times the FP32
 // rounding (about 1e-3 relative at 1M points), which cost the outer Krylov
 // solve ~20 % more iterations; in FP64 the cost is ~8 FP64 FMAs per lane.
-template <typename BOF>
-__device__ __forceinline__ float coarse_row(const AmgHeader& H, int64_t rho, BOF&& b_of) {
-    const int64_t nc = H.nc;
+// Right-hand sides (columns of B: [nc][Q]) two at a time, four partial sums a
+// lane and column (a DFMA's latency is 63 clocks), the lanes by the shared
+// butterfly: one at a time, in one chain, eight right-hand sides cost 23 us a
+// solve.  store(q, x) gets each column's x in one lane.
+template <int QT, typename T, typename Store>
+__device__ __forceinline__ void coarse_rows(const AmgHeader& H, int64_t rho, const T* B, int Q, Store&& store) {
+    constexpr int C = QT < 2 ? 1 : 2;       // columns at once
+    constexpr int kBatch = C == 1 ? 8 : 4;  // loads in flight a lane (and column)
+    const int nc = (int)H.nc, lane = (int)lane_id();
     const double* row = H.cinv64 + rho * nc;
-    double acc = 0.0;
-    for (int64_t c = lane_id(); c < nc; c += kWarp) acc = fma(row[c], (double)b_of(c), acc);
-    return (float)warp_sum(acc);
+#pragma unroll 1
+    for (int q0 = 0; q0 < QT && q0 < Q; q0 += C) {
+        double acc[4][C];
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+#pragma unroll
+            for (int p = 0; p < C; p++) acc[u][p] = 0.0;
+        for (int c0 = 0; c0 < nc; c0 += kBatch * kWarp) {
+            double w[kBatch];
+            T b[kBatch][C];
+#pragma unroll
+            for (int u = 0; u < kBatch; u++) {  // every load before the first use; past the end: the last column times 0
+                const int c = c0 + u * kWarp + lane;
+                const int cc = c < nc ? c : nc - 1;
+                w[u] = c < nc ? row[cc] : 0.0;
+#pragma unroll
+                for (int p = 0; p < C; p++) b[u][p] = q0 + p < Q ? B[(int64_t)cc * Q + q0 + p] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < kBatch; u++)
+                if (c0 + u * kWarp < nc)
+#pragma unroll
+                for (int p = 0; p < C; p++) acc[u % 4][p] = fma(w[u], (double)(float)b[u][p], acc[u % 4][p]);
+        }
+        double v[C];
+#pragma unroll
+        for (int p = 0; p < C; p++) v[p] = (acc[0][p] + acc[1][p]) + (acc[2][p] + acc[3][p]);
+        int q;
+        const float x = (float)warp_sum_multi<C>(v, lane, q);
+        if ((lane & (kWarp / C - 1)) == 0 && q0 + q < Q) store(q0 + q, x);
+    }
 }
 
 }  // namespace mvgd
