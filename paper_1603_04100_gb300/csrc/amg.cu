@@ -9,9 +9,9 @@
 //   * level l+1 is the Galerkin product P^T A_l P (entry (I, J) sums a_ij over
 //     the rows of aggregate I and the columns of aggregate J), computed in
 //     FP64 one warp per coarse row, with a fixed summation order;
-//   * the first level with at most kAmgCoarsest rows is inverted by
-//     Gauss-Jordan elimination with partial pivoting (FP32, one block),
-//     refined by two Newton-Schulz steps in FP64;
+//   * the first level with at most kAmgCoarsest rows is inverted by blocked
+//     Gauss-Jordan elimination with partial pivoting (FP32, a cluster of CTAs),
+//     refined by two Newton-Schulz steps to the FP64 level;
 //   * smoothing is a Jacobi step x += d (b - A x) with d_i = omega / a_ii on
 //     rows with a strong diagonal (a_ii > theta sum_j |a_ij|; omega = 0.9,
 //     theta = 0.3) and the l1 scaling d_i = 1 / sum_j |a_ij| (Baker, Falgout,
@@ -24,8 +24,9 @@
 #include <cooperative_groups.h>
 #include <limits.h>
 
-#include <algorithm>
 #include <string.h>
+
+#include <type_traits>
 
 #include "vcycle.cuh"
 
@@ -65,13 +66,12 @@ AmgLayout amg_layout(void* ws, int64_t n, int k) {
     }
     const int64_t nc = nlev > 0 ? sizes[nlev - 1] : 0;
     A.h.nc = nc;
-    A.h.dense = cv.take<float>(nc * nc);
     A.h.cinv = cv.take<float>(nc * nc);
-    A.h.piv = cv.take<int32_t>(nc);
     A.h.dense64 = cv.take<double>(nc * nc);
     A.h.cinv64 = cv.take<double>(nc * nc);
     A.h.ns_x = cv.take<double>(nc * nc);
     A.h.ns_t = cv.take<double>(nc * nc);
+    A.h.ns_s = cv.take<float>(2 * nc * nc);
     A.h.bytes = cv.used;
     return A;
 }
@@ -89,357 +89,655 @@ __device__ __forceinline__ double op_weight(const OpView& O, int64_t idx) {
                                : (double)static_cast<const float*>(O.val)[idx] + (double)O.val_lo[idx];
 }
 
+// The header, and the slice widths that the coarse levels collect, zeroed.
 __global__ void k_amg_header(AmgHeader h, AmgHeader* dst) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *dst = h;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, threads = (int64_t)gridDim.x * blockDim.x;
+    if (t == 0) *dst = h;
+    for (int l = 1; l < h.nlev; l++)
+        for (int64_t s = t; s < n_padded(h.lv[l].n) / kSlice; s += threads) h.lv[l].sw[s] = 0;
 }
 
 // Level 0: FP32 copy of the weights and the smoother's scaling of sigma I - L.
-__global__ void k_amg_level0(const AmgHeader* __restrict__ Hp, OpView O) {
+// Weights are loaded kLevel0Batch at a time before any is stored: stores to the
+// copy could alias the operator for all the compiler knows, and a load a slot
+// made the kernel a chain of K + 1 memory latencies.
+constexpr int kLevel0Batch = 7;
+__global__ void __launch_bounds__(256) k_amg_level0(const AmgHeader* __restrict__ Hp, OpView O) {
     const AmgHeader& H = *Hp;
     const int k = H.k, m = k + 1;
     const double sigma = H.sigma;
+    float* const out = H.lv[0].val;
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < H.n; r += (int64_t)gridDim.x * blockDim.x) {
         const int64_t vb = (r / kSlice) * (int64_t)(kSlice * m) + (r % kSlice);
         double l1 = 0.0, diag = 0.0;
-        for (int s = 0; s < m; s++) {
-            const int64_t idx = vb + (int64_t)s * kSlice;
-            const double w = op_weight(O, idx);
-            // FP64 weights round to nearest; the mixed format's hi is already that rounding
-            H.lv[0].val[idx] = O.prec == MVGD_FP64 ? (float)w : static_cast<const float*>(O.val)[idx];
-            if (s == 0) diag = sigma - w;
-            l1 += s == 0 ? fabs(sigma - w) : fabs(w);
+        for (int s0 = 0; s0 < m; s0 += kLevel0Batch) {
+            double w[kLevel0Batch];
+            float hi[kLevel0Batch];
+#pragma unroll
+            for (int u = 0; u < kLevel0Batch; u++) {
+                const int64_t idx = vb + (int64_t)(s0 + u < m ? s0 + u : s0) * kSlice;
+                if (O.prec == MVGD_FP64) {
+                    w[u] = static_cast<const double*>(O.val)[idx];
+                    hi[u] = (float)w[u];
+                } else {  // the mixed format's hi is already the weight's rounding
+                    hi[u] = static_cast<const float*>(O.val)[idx];
+                    w[u] = (double)hi[u] + (double)O.val_lo[idx];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kLevel0Batch; u++) {
+                if (s0 + u >= m) break;
+                out[vb + (int64_t)(s0 + u) * kSlice] = hi[u];
+                if (s0 + u == 0) diag = sigma - w[u];
+                l1 += s0 + u == 0 ? fabs(sigma - w[u]) : fabs(w[u]);
+            }
         }
         H.lv[0].dinv[r] = amg_smoother_scale(diag, l1);
     }
 }
 
-constexpr int kPerLane = kAmgAgg * kAmgStride / kWarp;  // entries a lane holds while coarsening
+// Row I of level l+1 by one warp, from the `total` entries of its aggregate's
+// rows: `fetch(e, key, v)` gives entry e < total (column aggregate and value),
+// PL of them a lane (entry t * 32 + lane).  Distinct columns come out in
+// increasing order, each with the FP64 sum of its entries: the lane's own in
+// entry order, then a butterfly over the warp, the same order on every run.
+//
+// FP64 instructions are what the kernel is bound by (an SM's FP64 pipe takes
+// one a warp in 16 clocks), then the search for the next column.  So each lane
+// first sorts its entries by (column, entry) and adds up its equal columns
+// once; columns are emitted kCoarsenGroup at a time, whose partial sums share
+// one butterfly (16 additions for 16 columns, 80 in separate ones, bit for bit
+// the same); and the row's l1 norm and sum gather in the lanes that end with
+// the totals.  Entries a lane is a template parameter because the sorting
+// network grows with its square: 15 exchanges for the 6 of K = 20 on level 0,
+// 120 for the 16 that a level of 64-entry rows can need.  All levels of
+// 1,048,576 rows, K = 20: 1.81 -> 0.82 ms, 0.71 ms of it level 1.
+constexpr int kCoarsenGroup = 16;
+template <int PL, typename Fetch>
+__device__ __forceinline__ void coarsen_row(const AmgHeader* Hp, const AmgLevel& Cl, int64_t I, int total,
+                                            Fetch&& fetch) {
+    const int lane = (int)lane_id();
+    int key[PL];
+    double v[PL];
+#pragma unroll
+    for (int t = 0; t < PL; t++) {
+        key[t] = INT_MAX;
+        v[t] = 0.0;
+        const int e = t * kWarp + lane;
+        if (e < total) fetch(e, key[t], v[t]);
+    }
+    // sort the lane's entries by (column, entry): an odd-even transposition network
+    int tt[PL];
+#pragma unroll
+    for (int t = 0; t < PL; t++) tt[t] = t;
+#pragma unroll
+    for (int ph = 0; ph < PL; ph++)
+#pragma unroll
+        for (int i = ph & 1; i + 1 < PL; i += 2) {
+            const bool sw = key[i] > key[i + 1] || (key[i] == key[i + 1] && tt[i] > tt[i + 1]);
+            const int ka = key[i], ta = tt[i];
+            const double va = v[i];
+            key[i] = sw ? key[i + 1] : ka;
+            tt[i] = sw ? tt[i + 1] : ta;
+            v[i] = sw ? v[i + 1] : va;
+            key[i + 1] = sw ? ka : key[i + 1];
+            tt[i + 1] = sw ? ta : tt[i + 1];
+            v[i + 1] = sw ? va : v[i + 1];
+        }
+    // the lane's sum of each column, in entry order, left on its last entry
+#pragma unroll
+    for (int t = 1; t < PL; t++)
+        if (key[t] != INT_MAX && key[t] == key[t - 1]) {
+            v[t] = v[t - 1] + v[t];
+            key[t - 1] = INT_MAX;
+        }
+    const int64_t ob = (I / kSlice) * (int64_t)(kSlice * kAmgStride) + (I % kSlice);
+    int out = 0;
+    double l1 = 0.0, rsum = 0.0, diag = 0.0;  // this lane's columns
+    bool more = true;
+    while (more) {
+        double part[kCoarsenGroup];
+        int cols = 0, mycol = INT_MAX;  // columns of this group; the one whose total this lane ends with
+#pragma unroll
+        for (int c = 0; c < kCoarsenGroup; c++) {
+            part[c] = 0.0;
+            if (!more) continue;  // warp-uniform
+            int mine = INT_MAX;
+#pragma unroll
+            for (int t = 0; t < PL; t++) mine = min(mine, key[t]);
+            const int m = __reduce_min_sync(0xffffffffu, mine);
+            if (m == INT_MAX) {
+                more = false;
+                continue;
+            }
+            if (mine == m) {
+#pragma unroll
+                for (int t = 0; t < PL; t++)
+                    if (key[t] == m) {  // at most one entry of the lane holds column m now
+                        part[c] = v[t];
+                        key[t] = INT_MAX;
+                    }
+            }
+            if (lane / (kWarp / kCoarsenGroup) == c) mycol = m;
+            cols++;
+        }
+        if (cols == 0) break;
+        int chan;
+        const double tot = warp_sum_multi<kCoarsenGroup>(part, lane, chan);
+        // lanes 2c and 2c + 1 hold value c (the halves a lane keeps follow its bits from the top)
+        if (chan < cols && (lane & 1) == 0) {
+            const int pos = out + chan;
+            if (pos < kAmgStride) {
+                Cl.col[ob + (int64_t)pos * kSlice] = mycol;
+                Cl.val64[ob + (int64_t)pos * kSlice] = tot;
+                Cl.val[ob + (int64_t)pos * kSlice] = (float)tot;
+            }
+            l1 += fabs(tot);
+            rsum += tot;
+            if (mycol == (int)I) diag = tot;
+        }
+        out += cols;
+    }
+    l1 = warp_sum(l1);
+    rsum = warp_sum(rsum);
+    diag = warp_sum(diag);  // one lane's value, zeros elsewhere
+    if (lane == 0) {
+        if (out > kAmgStride) atomicCAS((int*)&Hp->status, 0, (int)MVGD_EDEGENERATE);
+        if (out > *(volatile const int*)&Hp->width_max) atomicMax((int*)&Hp->width_max, out);
+        const int c = min(out, kAmgStride);
+        Cl.cnt[I] = c;
+        atomicMax(&Cl.sw[I / kSlice], c);  // the slice's widest row (zeroed with the header)
+        Cl.dinv[I] = amg_smoother_scale(diag, l1);
+        Cl.rs[I] = (float)rsum;
+    }
+    // padding: (own row, 0) up to the full stride, so slice loops need no bounds
+    for (int s = min(out, kAmgStride) + lane; s < kAmgStride; s += kWarp) {
+        Cl.col[ob + (int64_t)s * kSlice] = (int32_t)I;
+        Cl.val64[ob + (int64_t)s * kSlice] = 0.0;
+        Cl.val[ob + (int64_t)s * kSlice] = 0.0f;
+    }
+}
 
-// Level l+1 from level l, one warp per coarse row I: gather the entries of
-// the aggregate's rows, then emit distinct aggregate columns in increasing
-// order, each with the FP64 sum of its entries (per-lane sums in entry order,
-// then a butterfly over the warp: the same order on every run).  Each lane
-// first sorts its entries by (column, slot) and adds up its equal columns
-// once, so the merge over columns moves values instead of adding them: the
-// GPU's FP64 rate made those predicated adds (one per entry and column) the
-// kernel's cost.
-__global__ void k_amg_coarsen(const AmgHeader* Hp, OpView O, int l) {
+// Level 1 from the operator: every row has its K + 1 weights, so PL >= 8 (K + 1) / 32.
+template <int PL>
+__global__ void __launch_bounds__(256) k_amg_coarsen0(const AmgHeader* Hp, OpView O) {
+    const AmgHeader& H = *Hp;
+    const AmgLevel& Cl = H.lv[1];
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x / kWarp);
+    const int64_t n = H.lv[0].n;
+    const int k = H.k, W = k + 1;
+    for (int64_t I = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kWarp; I < Cl.n; I += warps) {
+        const int rows = (int)(n - I * kAmgAgg < kAmgAgg ? n - I * kAmgAgg : kAmgAgg);
+        coarsen_row<PL>(Hp, Cl, I, rows * W, [&](int e, int& key, double& v) {
+            const int f = e / W, s = e % W;
+            const int64_t i = I * kAmgAgg + f;
+            const double w = op_weight(O, (i / kSlice) * (int64_t)(kSlice * W) + (int64_t)s * kSlice + (i % kSlice));
+            if (s == 0) {
+                key = (int)I;
+                v = H.sigma - w;
+            } else {
+                const int64_t j = O.col[(i / kSlice) * (int64_t)(kSlice * k) + (int64_t)(s - 1) * kSlice + (i % kSlice)];
+                key = (int)(j / kAmgAgg);
+                v = -w;
+            }
+        });
+    }
+}
+
+// Level l+1 from level l >= 1: the rows' entries back to back, as many a lane
+// as they need (rows hold 10 to 25 entries typically, 64 at most).
+__global__ void __launch_bounds__(256) k_amg_coarsen(const AmgHeader* Hp, int l) {
     const AmgHeader& H = *Hp;
     const AmgLevel& F = H.lv[l];
     const AmgLevel& Cl = H.lv[l + 1];
     const int lane = (int)lane_id();
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x / kWarp);
-    const int k = H.k;
-    const int W = (l == 0) ? k + 1 : kAmgStride;  // entry slots per fine row
     for (int64_t I = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kWarp; I < Cl.n; I += warps) {
-        int key[kPerLane];
-        double v[kPerLane];
+        const int64_t mine = I * kAmgAgg + lane;
+        int end = lane < kAmgAgg && mine < F.n ? F.cnt[mine] : 0;  // inclusive prefix of the rows' counts
 #pragma unroll
-        for (int t = 0; t < kPerLane; t++) {
-            key[t] = INT_MAX;
-            v[t] = 0.0;
-            const int e = t * kWarp + lane;
-            const int f = e / W, s = e % W;
+        for (int o = 1; o < kAmgAgg; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += t;
+        }
+        int ends[kAmgAgg];
+#pragma unroll
+        for (int f = 0; f < kAmgAgg; f++) ends[f] = __shfl_sync(0xffffffffu, end, f);
+        const int total = ends[kAmgAgg - 1];
+        auto fetch = [&](int e, int& key, double& v) {
+            int f = 0, s = e;
+#pragma unroll
+            for (int g = 0; g + 1 < kAmgAgg; g++)
+                if (e >= ends[g]) {
+                    f = g + 1;
+                    s = e - ends[g];
+                }
             const int64_t i = I * kAmgAgg + f;
-            if (f >= kAmgAgg || i >= F.n) continue;
-            if (l == 0) {
-                const int64_t vb = (i / kSlice) * (int64_t)(kSlice * (k + 1)) + (i % kSlice);
-                const double w = op_weight(O, vb + (int64_t)s * kSlice);
-                if (s == 0) {
-                    key[t] = (int)(i / kAmgAgg);
-                    v[t] = H.sigma - w;
-                } else {
-                    const int64_t j = O.col[(i / kSlice) * (int64_t)(kSlice * k) + (int64_t)(s - 1) * kSlice + (i % kSlice)];
-                    key[t] = (int)(j / kAmgAgg);
-                    v[t] = -w;
-                }
-            } else if (s < F.cnt[i]) {
-                const int64_t idx = (i / kSlice) * (int64_t)(kSlice * kAmgStride) + (int64_t)s * kSlice + (i % kSlice);
-                key[t] = F.col[idx] / kAmgAgg;
-                v[t] = F.val64[idx];
-            }
-        }
-        // sort the lane's entries by (column, slot): an odd-even transposition network
-        int tt[kPerLane];
-#pragma unroll
-        for (int t = 0; t < kPerLane; t++) tt[t] = t;
-#pragma unroll
-        for (int ph = 0; ph < kPerLane; ph++)
-#pragma unroll
-            for (int i = ph & 1; i + 1 < kPerLane; i += 2) {
-                const bool sw = key[i] > key[i + 1] || (key[i] == key[i + 1] && tt[i] > tt[i + 1]);
-                const int ka = key[i], ta = tt[i];
-                const double va = v[i];
-                key[i] = sw ? key[i + 1] : ka;
-                tt[i] = sw ? tt[i + 1] : ta;
-                v[i] = sw ? v[i + 1] : va;
-                key[i + 1] = sw ? ka : key[i + 1];
-                tt[i + 1] = sw ? ta : tt[i + 1];
-                v[i + 1] = sw ? va : v[i + 1];
-            }
-        // the lane's sum of each column, in slot order, left on its last entry
-#pragma unroll
-        for (int t = 1; t < kPerLane; t++)
-            if (key[t] != INT_MAX && key[t] == key[t - 1]) {
-                v[t] = v[t - 1] + v[t];
-                key[t - 1] = INT_MAX;
-            }
-        const int64_t ob = (I / kSlice) * (int64_t)(kSlice * kAmgStride) + (I % kSlice);
-        int out = 0;
-        double l1 = 0.0, rsum = 0.0, diag = 0.0;
-        while (true) {
-            int mine = INT_MAX;
-#pragma unroll
-            for (int t = 0; t < kPerLane; t++) mine = min(mine, key[t]);
-            int m = mine;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = min(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (m == INT_MAX) break;
-            double part = 0.0;  // at most one entry of the lane holds column m now
-#pragma unroll
-            for (int t = 0; t < kPerLane; t++)
-                if (key[t] == m) {
-                    part = v[t];
-                    key[t] = INT_MAX;
-                }
-            const double tot = warp_sum(part);
-            if (out < kAmgStride && lane == 0) {
-                Cl.col[ob + (int64_t)out * kSlice] = m;
-                Cl.val64[ob + (int64_t)out * kSlice] = tot;
-                Cl.val[ob + (int64_t)out * kSlice] = (float)tot;
-            }
-            l1 += fabs(tot);
-            rsum += tot;
-            if (m == I) diag = tot;
-            out++;
-        }
-        if (lane == 0) {
-            if (out > kAmgStride) atomicCAS((int*)&Hp->status, 0, (int)MVGD_EDEGENERATE);
-            atomicMax((int*)&Hp->width_max, out);
-            const int c = min(out, kAmgStride);
-            Cl.cnt[I] = c;
-            Cl.dinv[I] = amg_smoother_scale(diag, l1);
-            Cl.rs[I] = (float)rsum;
-        }
-        // padding: (own row, 0) up to the full stride, so slice loops need no bounds
-        for (int s = min(out, kAmgStride) + lane; s < kAmgStride; s += kWarp) {
-            Cl.col[ob + (int64_t)s * kSlice] = (int32_t)I;
-            Cl.val64[ob + (int64_t)s * kSlice] = 0.0;
-            Cl.val[ob + (int64_t)s * kSlice] = 0.0f;
-        }
+            const int64_t idx = (i / kSlice) * (int64_t)(kSlice * kAmgStride) + (int64_t)s * kSlice + (i % kSlice);
+            key = F.col[idx] / kAmgAgg;
+            v = F.val64[idx];
+        };
+        if (total <= 4 * kWarp) coarsen_row<4>(Hp, Cl, I, total, fetch);
+        else if (total <= 8 * kWarp) coarsen_row<8>(Hp, Cl, I, total, fetch);
+        else coarsen_row<kAmgAgg * kAmgStride / kWarp>(Hp, Cl, I, total, fetch);
     }
 }
 
-// Widest row of each 32-row slice of level l (>= 1).
-__global__ void k_amg_slice_width(const AmgHeader* __restrict__ Hp, int l) {
-    const AmgLevel& L = Hp->lv[l];
-    const int64_t ns = (L.n + kSlice - 1) / kSlice;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < ns; s += (int64_t)gridDim.x * blockDim.x) {
-        int w = 0;
-        for (int64_t r = s * kSlice; r < (s + 1) * kSlice && r < L.n; r++) w = max(w, L.cnt[r]);
-        L.sw[s] = w;
-    }
+// x as hi + lo FP32 words (48 bits).
+__device__ __forceinline__ float2 split_f2(double x) {
+    const float hi = (float)x;
+    return make_float2(hi, (float)(x - (double)hi));
 }
 
-// The coarsest level as dense FP32 and FP64 matrices (both zeroed first).
+// The coarsest level as a dense FP64 matrix and its hi + lo split (in ns_x), a warp a row.
 __global__ void k_amg_dense(const AmgHeader* __restrict__ Hp, OpView O) {
     const AmgHeader& H = *Hp;
-    const int m = H.nlev - 1;
-    const int64_t nc = H.nc;
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < nc; r += (int64_t)gridDim.x * blockDim.x) {
-        float* row = H.dense + r * nc;
-        double* row64 = H.dense64 + r * nc;
-        if (m == 0) {
-            const int k = H.k;
-            const int64_t vb = (r / kSlice) * (int64_t)(kSlice * (k + 1)) + (r % kSlice);
-            row64[r] = H.sigma - op_weight(O, vb);
-            row[r] = (float)row64[r];
-            for (int s = 0; s < k; s++) {
-                const int64_t j = O.col[(r / kSlice) * (int64_t)(kSlice * k) + (int64_t)s * kSlice + (r % kSlice)];
-                row64[j] = -op_weight(O, vb + (int64_t)(s + 1) * kSlice);
-                row[j] = (float)row64[j];
-            }
-        } else {
-            const AmgLevel& L = H.lv[m];
-            const int64_t b = (r / kSlice) * (int64_t)(kSlice * kAmgStride) + (r % kSlice);
-            for (int s = 0; s < L.cnt[r]; s++) {
-                const int64_t e = b + (int64_t)s * kSlice;
-                row64[L.col[e]] = L.val64[e];
-                row[L.col[e]] = L.val[e];
-            }
+    const int m = H.nlev - 1, lane = (int)lane_id();
+    const int64_t nc = H.nc, r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kWarp;
+    if (r >= nc) return;
+    double* row = H.dense64 + r * nc;
+    float2* row2 = reinterpret_cast<float2*>(H.ns_x) + r * nc;
+    for (int64_t c = lane; c < nc; c += kWarp) {
+        row[c] = 0.0;
+        row2[c] = make_float2(0.0f, 0.0f);
+    }
+    __syncwarp();
+    auto put = [&](int64_t c, double v) {
+        row[c] = v;
+        row2[c] = split_f2(v);
+    };
+    if (m == 0) {
+        if (lane != 0) return;  // a folded operator's columns may repeat: one after the other
+        const int k = H.k;
+        const int64_t vb = (r / kSlice) * (int64_t)(kSlice * (k + 1)) + (r % kSlice);
+        put(r, H.sigma - op_weight(O, vb));
+        for (int s = 0; s < k; s++) {
+            const int64_t j = O.col[(r / kSlice) * (int64_t)(kSlice * k) + (int64_t)s * kSlice + (r % kSlice)];
+            put(j, -op_weight(O, vb + (int64_t)(s + 1) * kSlice));
+        }
+    } else {
+        const AmgLevel& L = H.lv[m];
+        const int64_t b = (r / kSlice) * (int64_t)(kSlice * kAmgStride) + (r % kSlice);
+        for (int s = lane; s < L.cnt[r]; s += kWarp) {
+            const int64_t e = b + (int64_t)s * kSlice;
+            put(L.col[e], L.val64[e]);
         }
     }
 }
 
-// cinv64 = the FP32 inverse (column-major) in FP64, row-major.
-__global__ void k_amg_promote(const AmgHeader* __restrict__ Hp) {
-    const int64_t n = Hp->nc;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * n; e += (int64_t)gridDim.x * blockDim.x)
-        Hp->cinv64[e] = (double)Hp->cinv[(e % n) * n + e / n];
+// ---------------------------------------------------------------------------
+// Inverse of the coarsest level: Gauss-Jordan in place with partial pivoting
+// in FP32, blocked.  Rows are not swapped: step k takes the largest |a_ik| of
+// the rows not yet used as a pivot (the lowest row on ties), and the
+// permutation p_k is undone on the way out, (A^-1)[k][p_j] = B[p_k][j].
+//
+// Steps go by panels of kInvPanel columns.  A panel's steps touch only its own
+// columns; their effect on any other column is the product with the panel's
+// result, a_new[i] = (i a pivot of the panel ? 0 : a[i]) + sum_t panel[i][t]
+// a_old[p_t].  A cluster of up to 8 CTAs holds the matrix in shared memory, 64
+// columns a CTA (139 KB at 512 rows).  Four warps of the CTA that owns the
+// panel's columns do the steps without any other CTA: a thread holds the 32
+// panel values of up to four rows in registers, one barrier of 128 threads a step.
+// (With a row a thread, 16 warps each read the pivot row, 8 LDS.128 a step, and
+// a step took 1,600 clocks.)  Then every CTA applies the panel to its columns in
+// 8 x 8 register tiles.  So the cluster meets once a panel; a matrix cut by rows
+// met four times a step, which made a step 4 us.  110 rows 0.44 -> 0.08 ms, 256
+// rows 1.17 -> 0.26 ms, 512 rows about 2.5 -> 0.57 ms; the chain of a step (two
+// warp reductions, the candidate row through shared memory, a reciprocal, one
+// register update a row) still takes about 1 us.
+// ---------------------------------------------------------------------------
+constexpr int kInvCols = 64;                // columns a CTA
+constexpr int kInvStride = kInvCols + 4;    // row stride: float4 accesses of consecutive rows hit all banks
+constexpr int kInvPanel = 32;
+constexpr int kInvThreads = 256;
+constexpr int kInvStepThreads = 128;        // threads that do a panel's steps
+
+// Rows of the panel's result, transposed [kInvPanel][pitch]; also the exchange
+// area in global memory (set-up scratch), followed by the pivots and a flag.
+__host__ __device__ constexpr int inv_pitch(int n) { return (n + 7) / 8 * 8; }
+__host__ __device__ constexpr size_t inv_panel_floats(int n) { return (size_t)inv_pitch(n) * kInvPanel + 64; }
+constexpr size_t inv_smem_floats(int n) {
+    return (size_t)n * kInvStride + (size_t)inv_pitch(n) * kInvPanel + kInvPanel * kInvCols;
 }
 
-// C = diag I + scale (A B) for small n x n row-major FP64 matrices: one block
-// per 32 x 32 tile of C, 32-wide k tiles staged in shared memory.  A Newton-
-// Schulz step X <- X (2I - A X) is two of these.
-constexpr int kGemmTile = 32;
-__global__ void __launch_bounds__(256) k_amg_dgemm(int n, const double* __restrict__ A, const double* __restrict__ B,
-                                                   double* __restrict__ Cm, double diag, double scale) {
-    __shared__ double As[kGemmTile][kGemmTile + 1], Bs[kGemmTile][kGemmTile + 1];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8 threads, 4 rows each
-    const int row0 = blockIdx.y * kGemmTile, col = blockIdx.x * kGemmTile + tx;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int k0 = 0; k0 < n; k0 += kGemmTile) {
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const int r = ty + 8 * u;
-            As[r][tx] = (row0 + r < n && k0 + tx < n) ? A[(int64_t)(row0 + r) * n + k0 + tx] : 0.0;
-            Bs[r][tx] = (k0 + r < n && col < n) ? B[(int64_t)(k0 + r) * n + col] : 0.0;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int kk = 0; kk < kGemmTile; kk++) {
-            const double b = Bs[kk][tx];
-#pragma unroll
-            for (int u = 0; u < 4; u++) acc[u] = fma(As[ty + 8 * u][kk], b, acc[u]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int u = 0; u < 4; u++) {
-        const int r = row0 + ty + 8 * u;
-        if (r < n && col < n) Cm[(int64_t)r * n + col] = scale * acc[u] + (r == col ? diag : 0.0);
-    }
-}
-
-// Gauss-Jordan inversion in place with partial pivoting.  Step k picks the
-// largest |a_ik|, i >= k (lowest i on ties), swaps rows k and p, and replaces
-// a by the matrix of the eliminated system; the column swaps are undone in
-// reverse order at the end (the classical in-place form).
-constexpr int kInvThreads = 1024;
-constexpr int kInvWarps = kInvThreads / 32;
-
-// The matrix is held in shared memory: a cluster of up to 8 CTAs (one an
-// SM), CTA q holding rows q*rows .. q*rows + rows - 1 (rows * n * 4 bytes
-// <= 128 KB).  Each step the CTAs publish their column-k pivot candidate,
-// every CTA reads all of them through distributed shared memory and picks the
-// same pivot (largest magnitude, lowest row on a tie), the owners swap rows k
-// and p, every CTA copies the pivot row, and each eliminates its own rows.
-// One block sweeping a 256 KB matrix through L2 every step took about 2 ms
-// for 256 rows.
-__global__ void __launch_bounds__(kInvThreads) k_amg_invert_cluster(AmgHeader* Hp, int rows) {
+// kInvRows: rows a step thread holds, n <= kInvRows * kInvStepThreads.
+template <int kInvRows>
+__global__ void __launch_bounds__(kInvThreads) k_amg_invert(AmgHeader* Hp) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank(), ncta = (int)cl.num_blocks();
-    const int n = (int)Hp->nc;
-    extern __shared__ float smf[];
-    float* A = smf;               // [rows][n] this CTA's rows
-    float* rowk = A + rows * n;   // [n] the scaled pivot row
-    float* tmp = rowk + n;        // [n] a row arriving in a swap
-    __shared__ float bv[kInvWarps], cand_v;
-    __shared__ int bi[kInvWarps], cand_i, piv_k, bad;
-    __shared__ int col_of[kAmgCoarsest];
+    const int n = (int)Hp->nc, pitch = inv_pitch(n);
+    extern __shared__ __align__(16) float smf[];
+    float* A = smf;                                    // [n][kInvStride] this CTA's columns
+    float* Pn = A + (size_t)n * kInvStride;            // [kInvPanel][pitch] the panel's result
+    float* U = Pn + (size_t)pitch * kInvPanel;         // [kInvPanel][kInvCols] the pivot rows before it
+    constexpr int kStepWarps = kInvStepThreads / kWarp;
+    __shared__ __align__(16) float cand[2][kStepWarps][kInvPanel];  // each warp's candidate row
+    __shared__ unsigned cand_key[2][kStepWarps];
+    __shared__ int cand_row[2][kStepWarps];
+    __shared__ int piv[kAmgCoarsest];       // pivot row of step k
+    __shared__ int panel_of[kAmgCoarsest];  // panel in which a row was the pivot
+    __shared__ int failed;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int r0 = rank * rows, r1 = min(n, r0 + rows);
-    float* a = Hp->dense;
-    for (int e = tid; e < (r1 - r0) * n; e += kInvThreads) A[e] = a[(int64_t)r0 * n + e];
-    if (tid == 0) bad = 0;
-    cl.sync();
-    for (int k = 0; k < n; k++) {
-        // this CTA's pivot candidate in column k
-        float best = -1.0f;
-        int bidx = INT_MAX;
-        for (int i = max(k, r0) + tid; i < r1; i += kInvThreads) {
-            const float v = fabsf(A[(i - r0) * n + k]);
-            if (v > best) { best = v; bidx = i; }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
-            if (ov > best || (ov == best && oi < bidx)) { best = ov; bidx = oi; }
-        }
-        if (lane == 0) { bv[wid] = best; bi[wid] = bidx; }
-        __syncthreads();
-        if (tid == 0) {
-            float b = -1.0f;
-            int p = INT_MAX;
-            for (int w = 0; w < kInvWarps; w++)
-                if (bv[w] > b || (bv[w] == b && bi[w] < p)) { b = bv[w]; p = bi[w]; }
-            cand_v = b;
-            cand_i = p;
-        }
-        cl.sync();
-        // every CTA takes the same pivot from all candidates
-        if (tid == 0) {
-            float b = -1.0f;
-            int p = INT_MAX;
-            for (int q = 0; q < ncta; q++) {
-                const float v = *cl.map_shared_rank(&cand_v, q);
-                const int i = *cl.map_shared_rank(&cand_i, q);
-                if (v > b || (v == b && i < p)) { b = v; p = i; }
-            }
-            if (!(b > 0.0f) || !isfinite(b)) bad = 1;
-            piv_k = p == INT_MAX ? k : p;
-            if (rank == 0) Hp->piv[k] = piv_k;
-        }
-        __syncthreads();
-        if (bad) break;  // the same decision in every CTA
-        const int p = piv_k;
-        const int ok = k / rows, op = p / rows;
-        if (p != k) {  // rows k and p trade places: each owner fetches the other row first
-            if (rank == ok)
-                for (int j = tid; j < n; j += kInvThreads) tmp[j] = cl.map_shared_rank(A, op)[(p - op * rows) * n + j];
-            if (rank == op && op != ok)
-                for (int j = tid; j < n; j += kInvThreads) tmp[j] = cl.map_shared_rank(A, ok)[(k - ok * rows) * n + j];
-            if (rank == op && op == ok)
-                for (int j = tid; j < n; j += kInvThreads) {
-                    const float t = A[(k - r0) * n + j];
-                    A[(k - r0) * n + j] = A[(p - r0) * n + j];
-                    A[(p - r0) * n + j] = t;
-                }
-            cl.sync();
-            if (op != ok) {
-                if (rank == ok) for (int j = tid; j < n; j += kInvThreads) A[(k - r0) * n + j] = tmp[j];
-                if (rank == op) for (int j = tid; j < n; j += kInvThreads) A[(p - r0) * n + j] = tmp[j];
-            }
-            cl.sync();
-        }
-        // the pivot row, scaled, in every CTA
-        const float* src = cl.map_shared_rank(A, ok) + (k - ok * rows) * n;
-        const float inv = 1.0f / src[k];
-        for (int j = tid; j < n; j += kInvThreads) rowk[j] = (j == k) ? inv : src[j] * inv;
-        cl.sync();  // every CTA has its copy before the owner overwrites row k
-        for (int i = r0 + wid; i < r1; i += kInvWarps) {
-            float* row = A + (i - r0) * n;
-            if (i == k) {
-                for (int j = lane; j < n; j += 32) row[j] = rowk[j];
-            } else {
-                const float cik = row[k];
-#pragma unroll 4
-                for (int j = lane; j < n; j += 32) row[j] = (j == k) ? -cik * inv : fmaf(-cik, rowk[j], row[j]);
-            }
-        }
-        __syncthreads();
+    const int c0 = rank * kInvCols, ncols = min(kInvCols, n - c0);
+    float* const xch = reinterpret_cast<float*>(Hp->ns_t);
+    for (int e = tid; e < n * kInvCols; e += kInvThreads) {
+        const int r = e / kInvCols, j = e % kInvCols;
+        A[r * kInvStride + j] = j < ncols ? (float)Hp->dense64[(int64_t)r * n + c0 + j] : 0.0f;
     }
-    if (bad) {
+    for (int r = tid; r < n; r += kInvThreads) panel_of[r] = -1;
+    if (tid == 0) failed = 0;
+    __syncthreads();
+    for (int p = 0; p * kInvPanel < n; p++) {
+        const int k0 = p * kInvPanel, kb = min(kInvPanel, n - k0), owner = k0 / kInvCols, lk = k0 % kInvCols;
+        float* const buf = xch + (p & 1) * inv_panel_floats(n);
+        int* const bufi = reinterpret_cast<int*>(buf + (size_t)pitch * kInvPanel);
+        if (rank == owner && tid < kInvStepThreads) {
+            float v[kInvRows][kInvPanel];
+            bool used[kInvRows];
+#pragma unroll
+            for (int q = 0; q < kInvRows; q++) {
+                const int i = tid + q * kInvStepThreads;
+                used[q] = i >= n || panel_of[i] >= 0;  // a row past the end is never a pivot
+#pragma unroll
+                for (int j = 0; j < kInvPanel; j += 4) {
+                    const float4 t = i < n ? *reinterpret_cast<const float4*>(A + i * kInvStride + lk + j)
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[q][j] = t.x; v[q][j + 1] = t.y; v[q][j + 2] = t.z; v[q][j + 3] = t.w;
+                }
+            }
+            bool bad = false;
+            // step t works on v[.][0] and turns the registers by one place: the loop is one body
+#pragma unroll 1
+            for (int t = 0; t < kInvPanel; t++) {
+                if (t >= kb || bad) {  // uniform over the step threads: past the last column (zeros), only turn
+#pragma unroll
+                    for (int q = 0; q < kInvRows; q++) {
+                        const float first = v[q][0];
+#pragma unroll
+                        for (int j = 0; j + 1 < kInvPanel; j++) v[q][j] = v[q][j + 1];
+                        v[q][kInvPanel - 1] = first;
+                    }
+                    continue;
+                }
+                const int b = t & 1;
+                unsigned key = 0u;
+                int mq = -1;  // this thread's candidate: its largest unused |v[.][0]|, the lowest row on ties
+#pragma unroll
+                for (int q = 0; q < kInvRows; q++) {
+                    const unsigned kq = __float_as_uint(fabsf(v[q][0]));
+                    if (!used[q] && (mq < 0 || kq > key)) { key = kq; mq = q; }
+                }
+                const unsigned wm = __reduce_max_sync(0xffffffffu, key);
+                const int row_of = mq >= 0 && key == wm ? tid + mq * kInvStepThreads : INT_MAX;
+                const int wr = __reduce_min_sync(0xffffffffu, row_of);
+                if (row_of == wr && wr != INT_MAX) {
+#pragma unroll
+                    for (int q = 0; q < kInvRows; q++)
+                        if (q == mq) {
+#pragma unroll
+                            for (int j = 0; j < kInvPanel; j += 4)
+                                *reinterpret_cast<float4*>(&cand[b][wid][j]) =
+                                    make_float4(v[q][j], v[q][j + 1], v[q][j + 2], v[q][j + 3]);
+                        }
+                }
+                if (lane == 0) {
+                    cand_key[b][wid] = wr == INT_MAX ? 0u : wm;
+                    cand_row[b][wid] = wr;
+                }
+                asm volatile("bar.sync 1, %0;" ::"n"(kInvStepThreads) : "memory");
+                unsigned m = cand_key[b][0];
+                int pr = cand_row[b][0], w = 0;
+#pragma unroll
+                for (int o = 1; o < kStepWarps; o++) {
+                    const unsigned ko = cand_key[b][o];
+                    const int ro = cand_row[b][o];
+                    if (ko > m || (ko == m && ro < pr)) { m = ko; pr = ro; w = o; }
+                }
+                if (m == 0u || m >= 0x7f800000u) {  // no pivot, or one that is not finite
+                    bad = true;
+                    t--;  // turn the rest of the way
+                    continue;
+                }
+                const float* row = cand[b][w];
+                const float inv = 1.0f / row[0];
+                float f[kInvRows];
+#pragma unroll
+                for (int q = 0; q < kInvRows; q++) f[q] = v[q][0] * inv;
+                // every row but the pivot: v - f x
+#pragma unroll
+                for (int j = 0; j < kInvPanel; j += 4) {
+                    const float4 x = *reinterpret_cast<const float4*>(row + j);
+#pragma unroll
+                    for (int q = 0; q < kInvRows; q++) {
+                        if (j > 0) v[q][j - 1] = fmaf(-f[q], x.x, v[q][j]);
+                        v[q][j] = fmaf(-f[q], x.y, v[q][j + 1]);
+                        v[q][j + 1] = fmaf(-f[q], x.z, v[q][j + 2]);
+                        v[q][j + 2] = fmaf(-f[q], x.w, v[q][j + 3]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < kInvRows; q++) v[q][kInvPanel - 1] = -f[q];
+                if ((pr & (kInvStepThreads - 1)) == tid) {  // the pivot row: x inv
+#pragma unroll
+                    for (int q = 0; q < kInvRows; q++)
+                        if (pr == tid + q * kInvStepThreads) {
+                            used[q] = true;
+#pragma unroll
+                            for (int j = 0; j + 1 < kInvPanel; j++) v[q][j] = row[j + 1] * inv;
+                            v[q][kInvPanel - 1] = inv;
+                        }
+                }
+                if (tid == 0) piv[k0 + t] = pr;
+            }
+#pragma unroll
+            for (int q = 0; q < kInvRows; q++) {
+                const int i = tid + q * kInvStepThreads;
+                if (i >= n) continue;
+#pragma unroll
+                for (int j = 0; j < kInvPanel; j++) {
+                    Pn[j * pitch + i] = v[q][j];
+                    if (ncta > 1) buf[j * pitch + i] = v[q][j];
+                }
+#pragma unroll
+                for (int j = 0; j < kInvPanel; j += 4)
+                    *reinterpret_cast<float4*>(A + i * kInvStride + lk + j) =
+                        make_float4(v[q][j], v[q][j + 1], v[q][j + 2], v[q][j + 3]);
+            }
+            asm volatile("bar.sync 1, %0;" ::"n"(kInvStepThreads) : "memory");  // piv
+            if (ncta > 1) {
+                if (tid < kb) bufi[tid] = bad ? 0 : piv[k0 + tid];
+                if (tid == 0) bufi[kInvPanel] = bad;
+            }
+            if (tid == 0) failed = bad;
+        }
+        if (ncta > 1) {
+            cl.sync();  // the panel is in global memory (its buffer was last read two panels ago)
+            if (rank != owner) {
+                for (int e = tid; e < pitch * kInvPanel / 4; e += kInvThreads)
+                    reinterpret_cast<float4*>(Pn)[e] = __ldcg(reinterpret_cast<const float4*>(buf) + e);
+                if (tid < kb) piv[k0 + tid] = __ldcg(bufi + tid);
+                if (tid == 0) failed = __ldcg(bufi + kInvPanel);
+            }
+        }
+        __syncthreads();
+        if (failed) break;  // the same decision in every CTA
+        if (tid < kb) panel_of[piv[k0 + tid]] = p;
+        for (int e = tid; e < kInvPanel * kInvCols; e += kInvThreads) {
+            const int t = e / kInvCols, j = e % kInvCols;
+            U[e] = t < kb ? A[piv[k0 + t] * kInvStride + j] : 0.0f;
+        }
+        __syncthreads();
+        for (int tile = tid; tile < pitch / 8 * (kInvCols / 8); tile += kInvThreads) {
+            const int rg = tile / (kInvCols / 8) * 8, cg8 = tile % (kInvCols / 8) * 8;
+            if (cg8 >= ncols || (rank == owner && cg8 >= lk && cg8 < lk + kInvPanel)) continue;
+            float acc[8][8];
+#pragma unroll
+            for (int r = 0; r < 8; r++) {
+                const int i = rg + r;
+                const bool old = i < n && panel_of[i] != p;
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const float4 t = old ? *reinterpret_cast<const float4*>(A + i * kInvStride + cg8 + 4 * h)
+                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+                    acc[r][4 * h] = t.x; acc[r][4 * h + 1] = t.y; acc[r][4 * h + 2] = t.z; acc[r][4 * h + 3] = t.w;
+                }
+            }
+#pragma unroll 2
+            for (int t = 0; t < kInvPanel; t++) {
+                const float4 u0 = *reinterpret_cast<const float4*>(U + t * kInvCols + cg8);
+                const float4 u1 = *reinterpret_cast<const float4*>(U + t * kInvCols + cg8 + 4);
+                const float4 x0 = *reinterpret_cast<const float4*>(Pn + t * pitch + rg);
+                const float4 x1 = *reinterpret_cast<const float4*>(Pn + t * pitch + rg + 4);
+                const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+                for (int r = 0; r < 8; r++) {
+                    acc[r][0] = fmaf(x[r], u0.x, acc[r][0]); acc[r][1] = fmaf(x[r], u0.y, acc[r][1]);
+                    acc[r][2] = fmaf(x[r], u0.z, acc[r][2]); acc[r][3] = fmaf(x[r], u0.w, acc[r][3]);
+                    acc[r][4] = fmaf(x[r], u1.x, acc[r][4]); acc[r][5] = fmaf(x[r], u1.y, acc[r][5]);
+                    acc[r][6] = fmaf(x[r], u1.z, acc[r][6]); acc[r][7] = fmaf(x[r], u1.w, acc[r][7]);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < 8; r++) {
+                if (rg + r >= n) continue;  // (the panel's columns past n hold whatever was there)
+                float* d = A + (rg + r) * kInvStride + cg8;
+                *reinterpret_cast<float4*>(d) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+                *reinterpret_cast<float4*>(d + 4) = make_float4(acc[r][4], acc[r][5], acc[r][6], acc[r][7]);
+            }
+        }
+        __syncthreads();  // this CTA's columns are up to date
+    }
+    if (failed) {
         if (rank == 0 && tid == 0) atomicCAS((int*)&Hp->status, 0, (int)MVGD_EDEGENERATE);
-        cl.sync();
         return;
     }
-    for (int e = tid; e < (r1 - r0) * n; e += kInvThreads) a[(int64_t)r0 * n + e] = A[e];
-    cl.sync();  // the rows of every CTA are in global memory
-    if (rank != 0) return;
-    if (tid == 0) {
-        for (int c = 0; c < n; c++) col_of[c] = c;
-        for (int k = n - 1; k >= 0; k--) {
-            const int p = Hp->piv[k], t = col_of[k];
-            col_of[k] = col_of[p];
-            col_of[p] = t;
+    // the pivots of every panel are in every CTA: the inverse in FP32, column-major
+    for (int e = tid; e < n * kInvCols; e += kInvThreads) {
+        const int j = e / n, k = e % n;
+        if (j >= ncols) continue;
+        Hp->cinv[(int64_t)piv[c0 + j] * n + k] = A[piv[k] * kInvStride + j];
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Newton-Schulz X <- X + X (I - A X), twice, which squares the FP32 inverse's
+// residual R = I - A X (~1e-5) each time, down to the FP64 level: four products
+// of small n x n matrices.
+//   kNsR0  R0 = I - A X0    A split into hi + lo FP32 words, X0 the FP32 inverse
+//   kNsX1  X1 = X0 + X0 R0  (FP64, and split)
+//   kNsR1  R1 = I - A X1    in FP64
+//   kNsX2  X2 = X1 + X1 R1  both split; the inverse that the cycle uses
+// The FP64 pipe takes 2 FMAs a clock an SM, so only the residual that decides
+// the final accuracy runs there.  The other products sum hi hi in compensated
+// FP32 arithmetic (f2_add_prod, about 2^-45 of sum |a||x|) with the cross terms
+// beside it, 11 FP32 instructions a term.  X R is a correction of 1e-5 of X and
+// less, so its error is below 2^-53 of X in the last step; in the first step the
+// error of R0 enters X2 squared.
+// A block of 4 warps takes a 16 x 16 tile (256 tiles at n = 256: more than SMs);
+// each warp takes every fourth group of 8 of the sum, 8 outputs a lane, and the
+// block adds the four partial sums.  All four: 317 -> 98 us at n = 256, of which
+// R1 43 us (27 at the FP64 pipe's rate).
+// ---------------------------------------------------------------------------
+enum NsStep : int { kNsR0 = 0, kNsX1 = 1, kNsR1 = 2, kNsX2 = 3 };
+constexpr int kNsTile = 16, kNsDeep = 32, kNsWarps = 4;
+
+template <int STEP>
+__global__ void __launch_bounds__(kNsWarps * kWarp) k_amg_ns(const AmgHeader* __restrict__ Hp) {
+    constexpr bool kFast = STEP != kNsR1;
+    using LT = typename std::conditional<STEP == kNsR1, double, typename std::conditional<STEP == kNsX1, float, float2>::type>::type;
+    using RT = typename std::conditional<STEP == kNsR1, double, typename std::conditional<STEP == kNsR0, float, float2>::type>::type;
+    using AT = typename std::conditional<kFast, F2, double>::type;
+    __shared__ LT Ls[kNsTile][kNsDeep + 1];
+    __shared__ RT Rs[kNsDeep][kNsTile + 1];
+    __shared__ AT sum[kNsWarps][kNsTile * kNsTile];
+    const AmgHeader& H = *Hp;
+    const int n = (int)H.nc;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int row0 = blockIdx.y * kNsTile, col0 = blockIdx.x * kNsTile;
+    const float* x0t = H.cinv;  // X0, column-major
+    auto left = [&](int r, int c) -> LT {
+        const int64_t e = (int64_t)r * n + c;
+        if constexpr (STEP == kNsR0) return reinterpret_cast<const float2*>(H.ns_x)[e];       // A
+        else if constexpr (STEP == kNsX1) return x0t[(int64_t)c * n + r];                     // X0
+        else if constexpr (STEP == kNsR1) return H.dense64[e];                                // A
+        else return reinterpret_cast<const float2*>(H.ns_s)[e];                               // X1
+    };
+    auto right = [&](int r, int c) -> RT {
+        const int64_t e = (int64_t)r * n + c;
+        if constexpr (STEP == kNsR0) return x0t[(int64_t)c * n + r];                          // X0
+        else if constexpr (STEP == kNsR1) return H.ns_x[e];                                   // X1
+        else return reinterpret_cast<const float2*>(H.ns_t)[e];                               // R0, R1
+    };
+    // lane: rows 2 (lane / 4) and the next, columns 4 (lane % 4) .. + 3
+    const int lr = 2 * (lane >> 2), lc = 4 * (lane & 3);
+    AT acc[2][4];
+#pragma unroll
+    for (int a = 0; a < 2; a++)
+#pragma unroll
+        for (int b = 0; b < 4; b++) acc[a][b] = AT{};
+    for (int k0 = 0; k0 < n; k0 += kNsDeep) {
+#pragma unroll
+        for (int e = tid; e < kNsTile * kNsDeep; e += kNsWarps * kWarp) {
+            // consecutive threads along the operand's contiguous index
+            const int r = STEP == kNsX1 ? e % kNsTile : e / kNsDeep, c = STEP == kNsX1 ? e / kNsTile : e % kNsDeep;
+            Ls[r][c] = row0 + r < n && k0 + c < n ? left(row0 + r, k0 + c) : LT{};
+            const int r2 = STEP == kNsR0 ? e % kNsDeep : e / kNsTile, c2 = STEP == kNsR0 ? e / kNsDeep : e % kNsTile;
+            Rs[r2][c2] = k0 + r2 < n && col0 + c2 < n ? right(k0 + r2, col0 + c2) : RT{};
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int kk = 0; kk < kNsDeep / kNsWarps; kk++) {
+            const int k = wid * (kNsDeep / kNsWarps) + kk;
+            LT x[2];
+            RT y[4];
+#pragma unroll
+            for (int a = 0; a < 2; a++) x[a] = Ls[lr + a][k];
+#pragma unroll
+            for (int b = 0; b < 4; b++) y[b] = Rs[k][lc + b];
+#pragma unroll
+            for (int a = 0; a < 2; a++)
+#pragma unroll
+                for (int b = 0; b < 4; b++) {
+                    if constexpr (STEP == kNsR1) {
+                        acc[a][b] = fma(x[a], y[b], acc[a][b]);
+                    } else if constexpr (STEP == kNsR0) {
+                        f2_add_prod(acc[a][b], x[a].x, y[b]);
+                        acc[a][b].lo = fmaf(x[a].y, y[b], acc[a][b].lo);
+                    } else if constexpr (STEP == kNsX1) {
+                        f2_add_prod(acc[a][b], x[a], y[b].x);
+                        acc[a][b].lo = fmaf(x[a], y[b].y, acc[a][b].lo);
+                    } else {
+                        f2_add_prod(acc[a][b], x[a].x, y[b].x);
+                        acc[a][b].lo = fmaf(x[a].x, y[b].y, fmaf(x[a].y, y[b].x, acc[a][b].lo));
+                    }
+                }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int a = 0; a < 2; a++)
+#pragma unroll
+        for (int b = 0; b < 4; b++) sum[wid][(lr + a) * kNsTile + lc + b] = acc[a][b];
+    __syncthreads();
+    for (int e = tid; e < kNsTile * kNsTile; e += kNsWarps * kWarp) {
+        const int r = row0 + e / kNsTile, c = col0 + e % kNsTile;
+        if (r >= n || c >= n) continue;
+        const AT t = part_add(part_add(sum[0][e], sum[1][e]), part_add(sum[2][e], sum[3][e]));
+        double s;
+        if constexpr (kFast) s = f2_to_double(t);
+        else s = t;
+        const int64_t o = (int64_t)r * n + c;
+        if constexpr (STEP == kNsR0 || STEP == kNsR1) {
+            reinterpret_cast<float2*>(H.ns_t)[o] = split_f2((r == c ? 1.0 : 0.0) - s);
+        } else if constexpr (STEP == kNsX1) {
+            const double x1 = (double)x0t[(int64_t)c * n + r] + s;
+            H.ns_x[o] = x1;
+            reinterpret_cast<float2*>(H.ns_s)[o] = split_f2(x1);
+        } else {
+            H.cinv64[o] = H.ns_x[o] + s;
         }
     }
-    __syncthreads();
-    for (int c = wid; c < n; c += kInvWarps)
-        for (int r = lane; r < n; r += 32) Hp->cinv[c * n + r] = a[r * n + col_of[c]];  // column-major
 }
 
 int grid_for(int64_t threads) {
@@ -575,24 +873,22 @@ MVGD_API mvgd_status mvgd_amg_setup(const mvgd_ell* L, double sigma, void* amg_w
     A.h.width_max = 0;
     cudaStream_t s = (cudaStream_t)stream;
     OpView O{L->col, L->val, L->val_lo, L->prec};
-    k_amg_header<<<1, 1, 0, s>>>(A.h, A.hdr);
+    k_amg_header<<<grid_for(n_padded(L->n) / kSlice / kAmgAgg + 1), 256, 0, s>>>(A.h, A.hdr);
     k_amg_level0<<<grid_for(L->n), 256, 0, s>>>(A.hdr, O);
     for (int l = 0; l + 1 < A.h.nlev; l++) {
-        const int64_t nc = A.h.lv[l + 1].n;
-        k_amg_coarsen<<<grid_for(nc * kWarp), 256, 0, s>>>(A.hdr, O, l);
-        k_amg_slice_width<<<grid_for(nc / kSlice + 1), 256, 0, s>>>(A.hdr, l + 1);
+        const int gb = grid_for(A.h.lv[l + 1].n * kWarp);
+        if (l > 0) k_amg_coarsen<<<gb, 256, 0, s>>>(A.hdr, l);
+        else if (L->k < 16) k_amg_coarsen0<4><<<gb, 256, 0, s>>>(A.hdr, O);
+        else if (L->k < 24) k_amg_coarsen0<6><<<gb, 256, 0, s>>>(A.hdr, O);
+        else k_amg_coarsen0<8><<<gb, 256, 0, s>>>(A.hdr, O);
     }
     const int64_t nc = A.h.nc;
-    MVGD_CUDA_TRY(cudaMemsetAsync(A.h.dense, 0, sizeof(float) * nc * nc, s));
-    MVGD_CUDA_TRY(cudaMemsetAsync(A.h.dense64, 0, sizeof(double) * nc * nc, s));
-    k_amg_dense<<<grid_for(nc), 256, 0, s>>>(A.hdr, O);
+    k_amg_dense<<<grid_for(nc * kWarp), 256, 0, s>>>(A.hdr, O);
     {
-        // rows a CTA holds: the matrix in at most 8 CTAs' shared memory (128 KB of rows each)
-        const int rows = (int)std::min<int64_t>(nc, 32768 / nc);
-        const int ncta = (int)((nc + rows - 1) / rows);
-        const size_t smem = sizeof(float) * ((size_t)rows * nc + 2 * nc);
-        MVGD_CUDA_TRY(cudaFuncSetAttribute(k_amg_invert_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem));
+        const int ncta = (int)((nc + kInvCols - 1) / kInvCols);
+        const size_t smem = sizeof(float) * inv_smem_floats((int)nc);
+        auto fn = nc <= kInvStepThreads ? k_amg_invert<1> : (nc <= 2 * kInvStepThreads ? k_amg_invert<2> : k_amg_invert<4>);
+        MVGD_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)ncta);
         cfg.blockDim = dim3(kInvThreads);
@@ -605,22 +901,13 @@ MVGD_API mvgd_status mvgd_amg_setup(const mvgd_ell* L, double sigma, void* amg_w
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        MVGD_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_amg_invert_cluster, A.hdr, rows));
+        MVGD_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, A.hdr));
     }
-    // two Newton-Schulz steps X <- X (2I - A X) in FP64 from the FP32 inverse: its
-    // residual (~1e-5) squares each step, to the FP64 level
-    k_amg_promote<<<grid_for(nc * nc), 256, 0, s>>>(A.hdr);
-    const dim3 gg((unsigned)((nc + kGemmTile - 1) / kGemmTile), (unsigned)((nc + kGemmTile - 1) / kGemmTile));
-    double* X = A.h.cinv64;
-    double* Xn = A.h.ns_x;
-    for (int step = 0; step < 2; step++) {
-        k_amg_dgemm<<<gg, 256, 0, s>>>((int)nc, A.h.dense64, X, A.h.ns_t, 2.0, -1.0);  // T = 2I - A X
-        k_amg_dgemm<<<gg, 256, 0, s>>>((int)nc, X, A.h.ns_t, Xn, 0.0, 1.0);          // X' = X T
-        double* t = X;
-        X = Xn;
-        Xn = t;
-    }
-    // after an even number of steps the result is back in cinv64
+    const dim3 gg((unsigned)((nc + kNsTile - 1) / kNsTile), (unsigned)((nc + kNsTile - 1) / kNsTile));
+    k_amg_ns<kNsR0><<<gg, kNsWarps * kWarp, 0, s>>>(A.hdr);
+    k_amg_ns<kNsX1><<<gg, kNsWarps * kWarp, 0, s>>>(A.hdr);
+    k_amg_ns<kNsR1><<<gg, kNsWarps * kWarp, 0, s>>>(A.hdr);
+    k_amg_ns<kNsX2><<<gg, kNsWarps * kWarp, 0, s>>>(A.hdr);
     return launch_status();
 }
 
