@@ -3,14 +3,14 @@
 // FP64 issues at 1/56 of the FP32 rate on this part, and a warp instruction
 // costs the same whether 1 or 32 lanes are active, so every FP64 step runs
 // lane-parallel over 32 independent points.  Each lane keeps its (k+1) x 7
-// design matrix [1, xi, eta, xi^2, xi eta, eta^2 | zeta] in shared memory,
-// laid out lane-contiguously (element e of lane l at e * 32 + l) so every
+// design matrix [1, xi, eta, xi^2, xi eta, eta^2 | zeta] in shared memory
+// (without the column of ones), laid out lane-contiguously (element e of lane l at e * 32 + l) so every
 // access is a conflict-free 256-byte wavefront.  One block = one warp = one
 // 32-row slice of the sliced ELL output, so every store is coalesced.
 //
 // Per point:
 //   offsets d_s = p_j - p_i of the k neighbours;
-//   barycenter and covariance of N(i); cyclic Jacobi -> e_x (largest),
+//   barycenter and covariance of N(i); its eigenvectors (eig3) -> e_x (largest),
 //   e_y (middle), e_z (smallest eigenvalue);
 //   h by the chosen rule; h-scaled local coordinates (xi, eta, zeta);
 //   Householder QR of the design matrix over p_i and N(i), applied to zeta;
@@ -28,7 +28,7 @@
 // kept for the eigenvectors of the 3x3 covariance:
 //   offsets p_j - p_i in FP64 (exact for nearby points), then split into
 //   double-float; barycenter, mean distance and covariance in double-float;
-//   an FP32 Jacobi frame polished by FP64 Jacobi sweeps on Q^T C Q;
+//   the frame in FP64 (eig3: FP32 Jacobi, FP64 finish);
 //   local coordinates centred at p_i and scaled by h in double-float;
 //   the least squares through the normal equations G = V^T V, formed from the
 //   double-float moments sum xi^a eta^b (a + b <= 4) and sum xi^a eta^b zeta,
@@ -44,6 +44,7 @@
 // refinement does not settle, or with a non-finite value or an invalid
 // neighbour index is handed to the FP64 path (k_assemble_fix), which also
 // sets its row_status.
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -54,6 +55,11 @@ namespace mvgd {
 namespace {
 
 constexpr int kCols = 7;
+
+// The FP32 path needs an overdetermined fit: with k < kMinKMixed the 6-unknown
+// fit over k + 1 points is square or nearly so, its conditioning is beyond
+// what double-float residuals settle, and the rows use FP64 arithmetic.
+constexpr int kMinKMixed = 8;
 
 struct AsmArgs {
     const double* pts;
@@ -84,9 +90,9 @@ __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
     extern __shared__ double sm[];
     const int lane = threadIdx.x & (kWarp - 1);
     const int k = A.k, m = k + 1;
-    double* smw = sm + (size_t)(threadIdx.x / kWarp) * (size_t)(A.kcap + 1) * kCols * kWarp;  // this warp's part
-    // element (r, c) of this lane's design matrix
-#define VM(r, c) smw[((r) * kCols + (c)) * kWarp + lane]
+    double* smw = sm + (size_t)(threadIdx.x / kWarp) * (size_t)(A.kcap + 1) * (kCols - 1) * kWarp;  // this warp's part
+    // element (r, c), c >= 1, of this lane's design matrix (first its offsets in c = 1, 2, 3)
+#define VM(r, c) smw[((r) * (kCols - 1) + (c) - 1) * kWarp + lane]
 
     const int64_t i = A.order ? (int64_t)A.order[row] : row;
     const double px = A.pts[3 * i], py = A.pts[3 * i + 1], pz = A.pts[3 * i + 2];
@@ -100,9 +106,9 @@ __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
         int64_t j = nb[s];
         if (j < 0 || j >= A.n) { idx_ok = false; j = i; }
         double dx = A.pts[3 * j] - px, dy = A.pts[3 * j + 1] - py, dz = A.pts[3 * j + 2] - pz;
-        VM(s + 1, 0) = dx;
-        VM(s + 1, 1) = dy;
-        VM(s + 1, 2) = dz;
+        VM(s + 1, 1) = dx;
+        VM(s + 1, 2) = dy;
+        VM(s + 1, 3) = dz;
         cx += dx; cy += dy; cz += dz;
     }
     const double rk = 1.0 / (double)k;
@@ -110,7 +116,7 @@ __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
     double C[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     double hsum = 0;
     for (int s = 0; s < k; s++) {
-        double dx = VM(s + 1, 0), dy = VM(s + 1, 1), dz = VM(s + 1, 2);
+        double dx = VM(s + 1, 1), dy = VM(s + 1, 2), dz = VM(s + 1, 3);
         if (s < A.delta_m) hsum += sqrt(dx * dx + dy * dy + dz * dz);
         dx -= cx; dy -= cy; dz -= cz;
         C[0][0] += dx * dx; C[0][1] += dx * dy; C[0][2] += dx * dz;
@@ -118,7 +124,11 @@ __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
     }
     C[1][0] = C[0][1]; C[2][0] = C[0][2]; C[2][1] = C[1][2];
     double V[3][3], ev[3];
-    jacobi3(C, V, ev);
+    // the plain sweeps where the fit is square or nearly so: such rows amplify the
+    // frame's rounding (K = 5 on a clustered cloud: 6e-11 of the row's largest weight
+    // off with them, 2e-10 with eig3, on its worst row)
+    if (k < kMinKMixed) jacobi3(C, V, ev);
+    else eig3(C, V, ev);
     int imax = 0, imin = 0;
     for (int a = 1; a < 3; a++) {
         if (ev[a] > ev[imax]) imax = a;
@@ -133,11 +143,11 @@ __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
     // local coordinates; quarter-range extents
     double x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
     for (int s = 1; s <= k; s++) {
-        double dx = VM(s, 0), dy = VM(s, 1), dz = VM(s, 2);
+        double dx = VM(s, 1), dy = VM(s, 2), dz = VM(s, 3);
         double lx = dx * ex0 + dy * ex1 + dz * ex2;
         double ly = dx * ey0 + dy * ey1 + dz * ey2;
         double lz = dx * ez0 + dy * ez1 + dz * ez2;
-        VM(s, 0) = lx; VM(s, 1) = ly; VM(s, 2) = lz;
+        VM(s, 1) = lx; VM(s, 2) = ly; VM(s, 3) = lz;
         x0 = fmin(x0, lx); x1 = fmax(x1, lx);
         y0 = fmin(y0, ly); y1 = fmax(y1, ly);
     }
@@ -146,47 +156,93 @@ __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
     h *= A.delta_scale;
     const double ih = 1.0 / h;
 
-    // design matrix in h units: row 0 is p_i itself
-    VM(0, 0) = 1.0;
-    for (int c = 1; c < kCols; c++) VM(0, c) = 0.0;
+    // design matrix in h units; row 0 is p_i itself, (1, 0, ..., 0), and column 0 all
+    // ones: neither is stored.  The column sums are the first reflection's products.
+    double sd[kCols];  // of the coming reflection: its products with columns c, then those times beta
+#pragma unroll
+    for (int c = 1; c < kCols; c++) sd[c] = 0.0;
     for (int s = 1; s <= k; s++) {
-        double xi = VM(s, 0) * ih, eta = VM(s, 1) * ih, zeta = VM(s, 2) * ih;
-        VM(s, 0) = 1.0; VM(s, 1) = xi; VM(s, 2) = eta;
-        VM(s, 3) = xi * xi; VM(s, 4) = xi * eta; VM(s, 5) = eta * eta;
-        VM(s, 6) = zeta;
+        const double xi = VM(s, 1) * ih, eta = VM(s, 2) * ih, zeta = VM(s, 3) * ih;
+        const double x[kCols] = {1.0, xi, eta, xi * xi, xi * eta, eta * eta, zeta};
+#pragma unroll
+        for (int c = 1; c < kCols; c++) {
+            VM(s, c) = x[c];
+            sd[c] += x[c];
+        }
     }
 
-    // Householder QR; v_k stored below the diagonal with v_k[k] kept in vk[k]
-    double rd[6], vk[6], bk[6];
-    for (int kc = 0; kc < 6; kc++) {
-        double sig = 0;
-        for (int r = kc; r < m; r++) { double a = VM(r, kc); sig += a * a; }
-        double xk = VM(kc, kc);
-        double alpha = (xk > 0) ? -sqrt(sig) : sqrt(sig);
-        double den = sig - xk * alpha;     // v^T v / 2
-        double beta = den > 0 ? 1.0 / den : 0.0;
-        double v0 = xk - alpha;
-        for (int c = kc + 1; c < kCols; c++) {
-            double sdot = v0 * VM(kc, c);
-            for (int r = kc + 1; r < m; r++) sdot += VM(r, kc) * VM(r, c);
-            sdot *= beta;
-            VM(kc, c) -= sdot * v0;
-            for (int r = kc + 1; r < m; r++) VM(r, c) -= sdot * VM(r, kc);
-        }
-        rd[kc] = alpha;
-        vk[kc] = v0;
-        bk[kc] = beta;
+    // Householder QR, v_k below the diagonal with v_k[k] in vk[k].  One pass over the
+    // rows a reflection: it is applied to the row's columns and the next one's norm and
+    // products are gathered on the way (column by column, two passes a column, the
+    // serial sums bound a launch of few rows and shared memory a full one).
+    double rd[6], vk[6], bk[6], ird[6];
+    {
+        const double sm1 = sqrt((double)m);  // column of ones: norm^2 m, x_0 = 1
+        rd[0] = -sm1;
+        vk[0] = 1.0 + sm1;
+        bk[0] = 1.0 / ((double)m + sm1);
+        ird[0] = -1.0 / sm1;
+#pragma unroll
+        for (int c = 1; c < kCols; c++) sd[c] *= bk[0];
+#pragma unroll
+        for (int c = 1; c < kCols; c++) VM(0, c) = -sd[c] * vk[0];
     }
+    auto reflect = [&](auto step) {  // applies reflection KC, forms reflection KC + 1
+        constexpr int KC = decltype(step)::value, N = KC + 1;
+        auto row = [&](int r, double (&x)[kCols]) {
+            const double a = KC == 0 ? 1.0 : VM(r, KC > 0 ? KC : 1);
+#pragma unroll
+            for (int c = N; c < kCols; c++) x[c] = fma(-sd[c], a, VM(r, c));
+        };
+        double top[kCols], g[kCols];
+        row(N, top);
+#pragma unroll
+        for (int c = N; c < kCols; c++) {
+            VM(N, c) = top[c];
+            g[c] = 0.0;
+        }
+        for (int r = N + 1; r < m; r++) {
+            double x[kCols];
+            row(r, x);
+#pragma unroll
+            for (int c = N; c < kCols; c++) {
+                VM(r, c) = x[c];
+                g[c] = fma(x[N], x[c], g[c]);
+            }
+        }
+        if constexpr (N < 6) {
+            const double xk = top[N], sig = fma(xk, xk, g[N]);
+            const double nrm = sqrt(sig), al = xk > 0 ? -nrm : nrm;
+            const double den = sig - xk * al;  // v^T v / 2
+            const double beta = den > 0 ? 1.0 / den : 0.0, v0 = xk - al;
+            rd[N] = al;
+            vk[N] = v0;
+            bk[N] = beta;
+            ird[N] = 1.0 / al;
+#pragma unroll
+            for (int c = N + 1; c < kCols; c++) {
+                sd[c] = beta * fma(v0, top[c], g[c]);
+                VM(N, c) = fma(-sd[c], v0, top[c]);  // row N of R
+            }
+        }
+    };
+    reflect(std::integral_constant<int, 0>{});
+    reflect(std::integral_constant<int, 1>{});
+    reflect(std::integral_constant<int, 2>{});
+    reflect(std::integral_constant<int, 3>{});
+    reflect(std::integral_constant<int, 4>{});  // (the fifth's only use left, row 5 of column 6, is formed above)
     double rmin = fabs(rd[0]);
     for (int c = 1; c < 6; c++) rmin = fmin(rmin, fabs(rd[c]));
     int st = (rmin < 1e-10 * fabs(rd[0])) ? 1 : 0;
 
     // a~ = R^-1 (Q^T zeta); only a~_1..a~_5 are needed
     double at[6];
+#pragma unroll
     for (int r = 5; r >= 1; r--) {
-        double s = VM(r, 6);
-        for (int c = r + 1; c < 6; c++) s -= VM(r, c) * at[c];
-        at[r] = s / rd[r];
+        double t = VM(r, 6);
+#pragma unroll
+        for (int c = r + 1; c < 6; c++) t -= VM(r, c) * at[c];
+        at[r] = t * ird[r];
     }
     const double zx = at[1], zy = at[2];
     const double zxx = 2.0 * at[3] * ih, zxy = at[4] * ih, zyy = 2.0 * at[5] * ih;
@@ -200,21 +256,49 @@ __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
     const double c0 = A.variant == MVGD_ROW_LS ? 0.0 : 2.0 * (A3 + A5);
     const double ct[6] = {c0, A1 * h, A2 * h, 2.0 * A3, A4, 2.0 * A5};
 
-    // t = R^-T c~ (forward substitution), y = Q [t; 0]
+    // t = R^-T c~ (forward substitution), y = Q [t; 0] in column 6
     double t[6];
+#pragma unroll
     for (int r = 0; r < 6; r++) {
-        double s = ct[r];
-        for (int c = 0; c < r; c++) s -= VM(c, r) * t[c];
-        t[r] = s / rd[r];
+        double u = ct[r];
+#pragma unroll
+        for (int c = 0; c < r; c++) u -= VM(c, r) * t[c];
+        t[r] = u * ird[r];
     }
-    for (int r = 0; r < m; r++) VM(r, 6) = (r < 6) ? t[r] : 0.0;
-    for (int kc = 5; kc >= 0; kc--) {
-        double sdot = vk[kc] * VM(kc, 6);
-        for (int r = kc + 1; r < m; r++) sdot += VM(r, kc) * VM(r, 6);
-        sdot *= bk[kc];
-        VM(kc, 6) -= sdot * vk[kc];
-        for (int r = kc + 1; r < m; r++) VM(r, 6) -= sdot * VM(r, kc);
+    for (int r = 0; r < m; r++) {
+        double v = 0.0;
+#pragma unroll
+        for (int c = 0; c < 6; c++) v = r == c ? t[c] : v;
+        VM(r, 6) = v;
     }
+    // reflections 5 .. 0: two partial sums each, the next one's products on the way
+    double part[2] = {0.0, 0.0};  // reflection 5's products with rows past its own: all zero yet
+    auto apply = [&](auto step) {
+        constexpr int KC = decltype(step)::value;
+        const double sdot = bk[KC] * fma(vk[KC], VM(KC, 6), part[0] + part[1]);
+        const double yk = fma(-sdot, vk[KC], VM(KC, 6));
+        VM(KC, 6) = yk;
+        part[0] = KC > 0 ? (KC == 1 ? yk : VM(KC, KC > 1 ? KC - 1 : 1) * yk) : 0.0;
+        part[1] = 0.0;
+        int r = KC + 1;
+        auto one = [&](int q, double& acc) {
+            const double a = KC == 0 ? 1.0 : VM(q, KC > 0 ? KC : 1);
+            const double y = fma(-sdot, a, VM(q, 6));
+            VM(q, 6) = y;
+            if (KC > 0) acc = fma(KC == 1 ? 1.0 : VM(q, KC > 1 ? KC - 1 : 1), y, acc);
+        };
+        for (; r + 1 < m; r += 2) {
+            one(r, part[0]);
+            one(r + 1, part[1]);
+        }
+        if (r < m) one(r, part[0]);
+    };
+    apply(std::integral_constant<int, 5>{});
+    apply(std::integral_constant<int, 4>{});
+    apply(std::integral_constant<int, 3>{});
+    apply(std::integral_constant<int, 2>{});
+    apply(std::integral_constant<int, 1>{});
+    apply(std::integral_constant<int, 0>{});
     const double ih2 = ih * ih;
     bool finite = isfinite(h) && h > 0;
     if (A.prec == MVGD_FP64) {
@@ -382,8 +466,8 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
     for (int s = 0; s < k; s++) {
         const int64_t j = nb[s];
         if (j < 0 || j >= A.n) return false;  // the FP64 path marks the row
-        const df dx = df_from_double(A.pts[3 * j] - px), dy = df_from_double(A.pts[3 * j + 1] - py),
-                 dz = df_from_double(A.pts[3 * j + 2] - pz);
+        const df dx = df_split(A.pts[3 * j] - px), dy = df_split(A.pts[3 * j + 1] - py),
+                 dz = df_split(A.pts[3 * j + 2] - pz);
         MF(s, 0) = dx.hi; MF(s, 1) = dx.lo;
         MF(s, 2) = dy.hi; MF(s, 3) = dy.lo;
         MF(s, 4) = dz.hi; MF(s, 5) = dz.lo;
@@ -401,37 +485,13 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
         C11 = df_fma(C11, ey, ey); C12 = df_fma(C12, ey, ez); C22 = df_fma(C22, ez, ez);
     }
 
-    // frame: FP32 Jacobi, its eigenvectors orthonormalised in FP64, the covariance
-    // rotated into them and finished by FP64 Jacobi sweeps (the FP64 eigen step)
+    // frame, in FP64 (the eigen step the mixed format keeps there)
     double E[3][3], ev[3];
     {
-        float Cf[3][3] = {{C00.hi, C01.hi, C02.hi}, {C01.hi, C11.hi, C12.hi}, {C02.hi, C12.hi, C22.hi}};
-        float Vf[3][3], wf[3];
-        jacobi3f(Cf, Vf, wf);
-        double Q[3][3];
-        for (int r = 0; r < 3; r++)
-            for (int c = 0; c < 3; c++) Q[r][c] = (double)Vf[r][c];
-        const double n0 = rsqrt(Q[0][0] * Q[0][0] + Q[1][0] * Q[1][0] + Q[2][0] * Q[2][0]);
-        for (int r = 0; r < 3; r++) Q[r][0] *= n0;
-        const double d01 = Q[0][0] * Q[0][1] + Q[1][0] * Q[1][1] + Q[2][0] * Q[2][1];
-        for (int r = 0; r < 3; r++) Q[r][1] -= d01 * Q[r][0];
-        const double n1 = rsqrt(Q[0][1] * Q[0][1] + Q[1][1] * Q[1][1] + Q[2][1] * Q[2][1]);
-        for (int r = 0; r < 3; r++) Q[r][1] *= n1;
-        Q[0][2] = Q[1][0] * Q[2][1] - Q[2][0] * Q[1][1];
-        Q[1][2] = Q[2][0] * Q[0][1] - Q[0][0] * Q[2][1];
-        Q[2][2] = Q[0][0] * Q[1][1] - Q[1][0] * Q[0][1];
-        const double C[3][3] = {{df_to_double(C00), df_to_double(C01), df_to_double(C02)},
-                                {df_to_double(C01), df_to_double(C11), df_to_double(C12)},
-                                {df_to_double(C02), df_to_double(C12), df_to_double(C22)}};
-        double T[3][3], B[3][3], W[3][3];
-        for (int r = 0; r < 3; r++)
-            for (int c = 0; c < 3; c++) T[r][c] = C[r][0] * Q[0][c] + C[r][1] * Q[1][c] + C[r][2] * Q[2][c];
-        for (int r = 0; r < 3; r++)
-            for (int c = r; c < 3; c++)
-                B[r][c] = B[c][r] = Q[0][r] * T[0][c] + Q[1][r] * T[1][c] + Q[2][r] * T[2][c];
-        jacobi3(B, W, ev);
-        for (int r = 0; r < 3; r++)
-            for (int c = 0; c < 3; c++) E[r][c] = Q[r][0] * W[0][c] + Q[r][1] * W[1][c] + Q[r][2] * W[2][c];
+        double C[3][3] = {{df_to_double(C00), df_to_double(C01), df_to_double(C02)},
+                          {0.0, df_to_double(C11), df_to_double(C12)},
+                          {0.0, 0.0, df_to_double(C22)}};
+        eig3(C, E, ev);
     }
     int imax = 0, imin = 0;
     for (int a = 1; a < 3; a++) {
@@ -440,9 +500,9 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
     }
     if (imax == imin) imin = (imax + 1) % 3;
     const int imid = 3 - imax - imin;
-    const df ex0 = df_from_double(E[0][imax]), ex1 = df_from_double(E[1][imax]), ex2 = df_from_double(E[2][imax]);
-    const df ey0 = df_from_double(E[0][imid]), ey1 = df_from_double(E[1][imid]), ey2 = df_from_double(E[2][imid]);
-    const df ez0 = df_from_double(E[0][imin]), ez1 = df_from_double(E[1][imin]), ez2 = df_from_double(E[2][imin]);
+    const df ex0 = df_split(E[0][imax]), ex1 = df_split(E[1][imax]), ex2 = df_split(E[2][imax]);
+    const df ey0 = df_split(E[0][imid]), ey1 = df_split(E[1][imid]), ey2 = df_split(E[2][imid]);
+    const df ez0 = df_split(E[0][imin]), ez1 = df_split(E[1][imin]), ez2 = df_split(E[2][imin]);
 
     // local coordinates centred at p_i; quarter-range extents
     df x0 = df_make(3e38f), x1 = df_make(-3e38f), y0 = x0, y1 = x1;
@@ -689,13 +749,8 @@ AsmWs asm_ws(void* base, int64_t n) {
     return w;
 }
 
-size_t smem_fp64(int k) { return sizeof(double) * (size_t)(k + 1) * kCols * kWarp; }
+size_t smem_fp64(int k) { return sizeof(double) * (size_t)(k + 1) * (kCols - 1) * kWarp; }
 size_t smem_mixed(int k) { return sizeof(float) * (size_t)k * kMixCols * kWarp; }
-
-// The FP32 path needs an overdetermined fit: with k < kMinKMixed the 6-unknown
-// fit over k + 1 points is square or nearly so, its conditioning is beyond
-// what double-float residuals settle, and the rows use FP64 arithmetic.
-constexpr int kMinKMixed = 8;
 
 bool fp32_path(const mvgd_ell& L, const mvgd_delta_rule& rule) {
     return L.prec == MVGD_FP32_REFINE && rule.arith == 0 && L.k >= kMinKMixed;
@@ -750,7 +805,7 @@ MVGD_API mvgd_status mvgd_assemble(const double* pts, int64_t n, int32_t k, cons
     if (L->order) k_invert_order<<<gb, 256, 0, s>>>(L->order, n, W.inv);
     const int64_t nslices = n_padded(n) / kSlice;
     // warps a block: the launch's tuning for the FP32 path (15 KB of shared memory a
-    // warp); the FP64 arithmetic keeps one (38 KB a warp: more would only cost
+    // warp); the FP64 arithmetic keeps one (32 KB a warp at K = 20: more would only cost
     // resident warps)
     int wpb = mixed ? tuned_assemble_warps() : 1;
     const size_t per_warp = mixed ? smem_mixed(k) : smem_fp64(k);
