@@ -84,6 +84,9 @@ struct AsmArgs {
     int32_t* nfix;
 };
 
+// isfinite by the exponent bits (a comparison of doubles runs on the FP64 pipe).
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
 // Stored row `row` of one cloud's operator in FP64, by this lane (its design
 // matrix lives in the lane's column of the warp's shared memory).
 __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
@@ -148,8 +151,10 @@ __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
         double ly = dx * ey0 + dy * ey1 + dz * ey2;
         double lz = dx * ez0 + dy * ez1 + dz * ez2;
         VM(s, 1) = lx; VM(s, 2) = ly; VM(s, 3) = lz;
-        x0 = fmin(x0, lx); x1 = fmax(x1, lx);
-        y0 = fmin(y0, ly); y1 = fmax(y1, ly);
+        if (A.delta_kind == MVGD_DELTA_QUARTER_RANGE) {  // (minima and maxima run on the FP64 pipe too)
+            x0 = fmin(x0, lx); x1 = fmax(x1, lx);
+            y0 = fmin(y0, ly); y1 = fmax(y1, ly);
+        }
     }
     double h = (A.delta_kind == MVGD_DELTA_QUARTER_RANGE) ? fmin(0.25 * (x1 - x0), 0.25 * (y1 - y0))
                                                           : hsum / (double)A.delta_m;
@@ -213,12 +218,12 @@ __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
         if constexpr (N < 6) {
             const double xk = top[N], sig = fma(xk, xk, g[N]);
             const double nrm = sqrt(sig), al = xk > 0 ? -nrm : nrm;
-            const double den = sig - xk * al;  // v^T v / 2
-            const double beta = den > 0 ? 1.0 / den : 0.0, v0 = xk - al;
+            const double v0 = xk - al, den = -al * v0;  // v^T v / 2 = sig - xk al
+            const double iden = 1.0 / den, beta = den > 0 ? iden : 0.0;
             rd[N] = al;
             vk[N] = v0;
             bk[N] = beta;
-            ird[N] = 1.0 / al;
+            ird[N] = -v0 * iden;  // 1 / al
 #pragma unroll
             for (int c = N + 1; c < kCols; c++) {
                 sd[c] = beta * fma(v0, top[c], g[c]);
@@ -305,14 +310,14 @@ __device__ __noinline__ void assemble_lane(const AsmArgs& A, int64_t row) {
         double* vo = static_cast<double*>(A.val);
         for (int r = 0; r < m; r++) {
             double w = (r == 0 ? VM(0, 6) - c0 : VM(r, 6)) * ih2;
-            finite = finite && isfinite(w);
+            finite = finite && finite64(w);
             vo[sell_index(row, r, m)] = w;
         }
     } else {
         float* vo = static_cast<float*>(A.val);
         for (int r = 0; r < m; r++) {
             double w = (r == 0 ? VM(0, 6) - c0 : VM(r, 6)) * ih2;
-            finite = finite && isfinite(w);
+            finite = finite && finite64(w);
             float hi = __double2float_rn(w);
             vo[sell_index(row, r, m)] = hi;
             A.val_lo[sell_index(row, r, m)] = __double2float_rn(w - (double)hi);
@@ -338,6 +343,7 @@ constexpr int kRefineSteps = 4;          // refinement steps of each 6x6 solve
 constexpr float kPivotFloor = 0x1p-16f;  // Cholesky pivot / diagonal below this: FP64 path
 constexpr float kCondCap = 4096.0f;      // 1-norm condition number of G above this: FP64 path
 constexpr float kSettled = 0x1p-30f;     // last correction / solution above this: FP64 path
+constexpr float kRefined = 0x1p-46f;     // correction / solution below this: no further step
 
 // Index of the moment sum xi^a eta^b (a + b <= 4) among the 15 moments.
 __host__ __device__ constexpr int moment_index(int a, int b) { return (a + b) * (a + b + 1) / 2 + b; }
@@ -347,9 +353,10 @@ __host__ __device__ constexpr int mono_b(int p) { return p == 2 || p == 4 ? 1 : 
 
 __host__ __device__ constexpr int tri(int i, int j) { return i * (i + 1) / 2 + j; }  // packed lower, j <= i
 
-// FP32 Cholesky G = L L^T of the hi parts of a symmetric 6x6 (packed lower).
-// False when a pivot falls below kPivotFloor of its diagonal entry.
-__device__ __forceinline__ bool chol6(const df (&G)[21], float (&L)[21]) {
+// FP32 Cholesky G = L L^T of the hi parts of a symmetric 6x6 (packed lower), the
+// diagonal of L inverted (il).  False when a pivot falls below kPivotFloor of its
+// diagonal entry.
+__device__ __forceinline__ bool chol6(const df (&G)[21], float (&L)[21], float (&il)[6]) {
     bool ok = true;
 #pragma unroll
     for (int j = 0; j < 6; j++) {
@@ -357,75 +364,76 @@ __device__ __forceinline__ bool chol6(const df (&G)[21], float (&L)[21]) {
 #pragma unroll
         for (int q = 0; q < j; q++) d = fmaf(-L[tri(j, q)], L[tri(j, q)], d);
         ok = ok && (d > kPivotFloor * G[tri(j, j)].hi);
-        const float ljj = sqrtf(fmaxf(d, 1e-30f));
-        L[tri(j, j)] = ljj;
-        const float inv = 1.0f / ljj;
+        il[j] = rsqrtf(fmaxf(d, 1e-30f));
 #pragma unroll
         for (int i = j + 1; i < 6; i++) {
             float t = G[tri(i, j)].hi;
 #pragma unroll
             for (int q = 0; q < j; q++) t = fmaf(-L[tri(i, q)], L[tri(j, q)], t);
-            L[tri(i, j)] = t * inv;
+            L[tri(i, j)] = t * il[j];
         }
     }
     return ok;
 }
 
 // x = (L L^T)^-1 r in FP32.
-__device__ __forceinline__ void chol6_solve(const float (&L)[21], const float (&r)[6], float (&x)[6]) {
+__device__ __forceinline__ void chol6_solve(const float (&L)[21], const float (&il)[6], const float (&r)[6],
+                                            float (&x)[6]) {
     float z[6];
 #pragma unroll
     for (int i = 0; i < 6; i++) {
         float t = r[i];
 #pragma unroll
         for (int q = 0; q < i; q++) t = fmaf(-L[tri(i, q)], z[q], t);
-        z[i] = t / L[tri(i, i)];
+        z[i] = t * il[i];
     }
 #pragma unroll
     for (int i = 5; i >= 0; i--) {
         float t = z[i];
 #pragma unroll
         for (int q = i + 1; q < 6; q++) t = fmaf(-L[tri(q, i)], x[q], t);
-        x[i] = t / L[tri(i, i)];
+        x[i] = t * il[i];
     }
 }
 
 // The 1-norm condition number |G|_1 |G^-1|_1 of the hi parts, G^-1 column by
 // column from the FP32 factor.  It sets the accuracy the double-float
 // residuals can reach, about cond(G) 2^-48 of the solution.
-__device__ __forceinline__ float cond1_6(const df (&G)[21], const float (&L)[21]) {
+__device__ __forceinline__ float cond1_6(const df (&G)[21], const float (&L)[21], const float (&il)[6]) {
     float gn = 0.0f, gin = 0.0f;
 #pragma unroll
     for (int j = 0; j < 6; j++) {
-        float e[6], x[6], cs = 0.0f, ci = 0.0f;
+        float cs = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 6; i++) {
-            e[i] = i == j ? 1.0f : 0.0f;
-            cs += fabsf(G[i >= j ? tri(i, j) : tri(j, i)].hi);
-        }
-        chol6_solve(L, e, x);
+        for (int i = 0; i < 6; i++) cs += fabsf(G[i >= j ? tri(i, j) : tri(j, i)].hi);
+        gn = fmaxf(gn, cs);
+    }
+#pragma unroll 1
+    for (int j = 0; j < 6; j++) {
+        float e[6], x[6], ci = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 6; i++) e[i] = i == j ? 1.0f : 0.0f;
+        chol6_solve(L, il, e, x);
 #pragma unroll
         for (int i = 0; i < 6; i++) ci += fabsf(x[i]);
-        gn = fmaxf(gn, cs);
         gin = fmaxf(gin, ci);
     }
     return gn * gin;
 }
 
-// Solves G x = rhs: the FP32 factor's solution, then kRefineSteps corrections
-// from double-float residuals rhs - G x.  False when the last correction is
-// still above kSettled of the solution (the factor does not contract).
-__device__ __forceinline__ bool solve6_refined(const df (&G)[21], const float (&L)[21], const df (&rhs)[6],
-                                               df (&x)[6]) {
-    float r[6], d[6];
+// Solves G x = rhs: corrections by the FP32 factor of double-float residuals rhs -
+// G x from x = 0 on, until one is below kRefined of the solution -- each shrinks by
+// the factor's contraction, 2^-12 at least, so the next would not be seen -- or
+// kRefineSteps after the first are done.  False when the last one is still above
+// kSettled (the factor does not contract).
+__device__ __forceinline__ bool solve6_refined(const df (&G)[21], const float (&L)[21], const float (&il)[6],
+                                               const df (&rhs)[6], df (&x)[6]) {
 #pragma unroll
-    for (int p = 0; p < 6; p++) r[p] = rhs[p].hi;
-    chol6_solve(L, r, d);
-#pragma unroll
-    for (int p = 0; p < 6; p++) x[p] = df_make(d[p]);
+    for (int p = 0; p < 6; p++) x[p] = df_make(0.0f);
     float last = 0.0f, xmax = 0.0f;
 #pragma unroll 1
-    for (int it = 0; it < kRefineSteps; it++) {
+    for (int it = 0; it <= kRefineSteps; it++) {
+        float r[6], d[6];
 #pragma unroll
         for (int p = 0; p < 6; p++) {
             df t = rhs[p];
@@ -433,7 +441,7 @@ __device__ __forceinline__ bool solve6_refined(const df (&G)[21], const float (&
             for (int q = 0; q < 6; q++) t = df_sub(t, df_mul(G[p >= q ? tri(p, q) : tri(q, p)], x[q]));
             r[p] = t.hi;
         }
-        chol6_solve(L, r, d);
+        chol6_solve(L, il, r, d);
         last = 0.0f;
         xmax = 0.0f;
 #pragma unroll
@@ -442,6 +450,7 @@ __device__ __forceinline__ bool solve6_refined(const df (&G)[21], const float (&
             last = fmaxf(last, fabsf(d[p]));
             xmax = fmaxf(xmax, fabsf(x[p].hi));
         }
+        if (last <= kRefined * xmax) break;
     }
     return last <= kSettled * xmax;
 }
@@ -462,7 +471,7 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
 
     // offsets d_s = p_j - p_i (FP64, then double-float), barycenter of N(i),
     // mean distance to the delta_m nearest
-    df cx = df_make(0.f), cy = df_make(0.f), cz = df_make(0.f), hsum = df_make(0.f);
+    df_acc sx = acc_zero(), sy = acc_zero(), sz = acc_zero(), hs = acc_zero();
     for (int s = 0; s < k; s++) {
         const int64_t j = nb[s];
         if (j < 0 || j >= A.n) return false;  // the FP64 path marks the row
@@ -471,26 +480,24 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
         MF(s, 0) = dx.hi; MF(s, 1) = dx.lo;
         MF(s, 2) = dy.hi; MF(s, 3) = dy.lo;
         MF(s, 4) = dz.hi; MF(s, 5) = dz.lo;
-        cx = df_add(cx, dx); cy = df_add(cy, dy); cz = df_add(cz, dz);
-        if (s < A.delta_m)
-            hsum = df_add(hsum, df_sqrt(df_add(df_add(df_mul(dx, dx), df_mul(dy, dy)), df_mul(dz, dz))));
+        acc_add(sx, dx); acc_add(sy, dy); acc_add(sz, dz);
+        if (s < A.delta_m) acc_add(hs, df_sqrt(df_dot3(dx, dx, dy, dy, dz, dz)));
     }
-    const df kk = df_make((float)k);
-    cx = df_div(cx, kk); cy = df_div(cy, kk); cz = df_div(cz, kk);
-    df C00 = df_make(0.f), C01 = C00, C02 = C00, C11 = C00, C12 = C00, C22 = C00;
+    const df kk = df_make((float)k), hsum = acc_value(hs);
+    const df cx = df_div(acc_value(sx), kk), cy = df_div(acc_value(sy), kk), cz = df_div(acc_value(sz), kk);
+    df_acc C00 = acc_zero(), C01 = C00, C02 = C00, C11 = C00, C12 = C00, C22 = C00;
     for (int s = 0; s < k; s++) {
         const df ex = df_sub({MF(s, 0), MF(s, 1)}, cx), ey = df_sub({MF(s, 2), MF(s, 3)}, cy),
                  ez = df_sub({MF(s, 4), MF(s, 5)}, cz);
-        C00 = df_fma(C00, ex, ex); C01 = df_fma(C01, ex, ey); C02 = df_fma(C02, ex, ez);
-        C11 = df_fma(C11, ey, ey); C12 = df_fma(C12, ey, ez); C22 = df_fma(C22, ez, ez);
+        acc_fma(C00, ex, ex); acc_fma(C01, ex, ey); acc_fma(C02, ex, ez);
+        acc_fma(C11, ey, ey); acc_fma(C12, ey, ez); acc_fma(C22, ez, ez);
     }
 
     // frame, in FP64 (the eigen step the mixed format keeps there)
     double E[3][3], ev[3];
     {
-        double C[3][3] = {{df_to_double(C00), df_to_double(C01), df_to_double(C02)},
-                          {0.0, df_to_double(C11), df_to_double(C12)},
-                          {0.0, 0.0, df_to_double(C22)}};
+        auto full = [](df_acc t) { return (double)t.hi + (double)t.lo; };
+        double C[3][3] = {{full(C00), full(C01), full(C02)}, {0.0, full(C11), full(C12)}, {0.0, 0.0, full(C22)}};
         eig3(C, E, ev);
     }
     int imax = 0, imin = 0;
@@ -508,16 +515,18 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
     df x0 = df_make(3e38f), x1 = df_make(-3e38f), y0 = x0, y1 = x1;
     for (int s = 0; s < k; s++) {
         const df dx = {MF(s, 0), MF(s, 1)}, dy = {MF(s, 2), MF(s, 3)}, dz = {MF(s, 4), MF(s, 5)};
-        const df lx = df_add(df_add(df_mul(dx, ex0), df_mul(dy, ex1)), df_mul(dz, ex2));
-        const df ly = df_add(df_add(df_mul(dx, ey0), df_mul(dy, ey1)), df_mul(dz, ey2));
-        const df lz = df_add(df_add(df_mul(dx, ez0), df_mul(dy, ez1)), df_mul(dz, ez2));
+        const df lx = df_dot3(dx, ex0, dy, ex1, dz, ex2);
+        const df ly = df_dot3(dx, ey0, dy, ey1, dz, ey2);
+        const df lz = df_dot3(dx, ez0, dy, ez1, dz, ez2);
         MF(s, 0) = lx.hi; MF(s, 1) = lx.lo;
         MF(s, 2) = ly.hi; MF(s, 3) = ly.lo;
         MF(s, 4) = lz.hi; MF(s, 5) = lz.lo;
-        if (df_less(lx, x0)) x0 = lx;
-        if (df_less(x1, lx)) x1 = lx;
-        if (df_less(ly, y0)) y0 = ly;
-        if (df_less(y1, ly)) y1 = ly;
+        if (A.delta_kind == MVGD_DELTA_QUARTER_RANGE) {
+            if (df_less(lx, x0)) x0 = lx;
+            if (df_less(x1, lx)) x1 = lx;
+            if (df_less(ly, y0)) y0 = ly;
+            if (df_less(y1, ly)) y1 = ly;
+        }
     }
     df h;
     if (A.delta_kind == MVGD_DELTA_QUARTER_RANGE) {
@@ -528,7 +537,9 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
     }
     h = df_mul(h, df_from_double(A.delta_scale));
     if (!(h.hi > 0.0f) || !df_isfinite(h)) return false;
-    const df ih = df_div(df_make(1.0f), h);
+    // 1 / h and its square once in FP64: the error of h^-2 is the whole row's
+    const double ihd = 1.0 / df_to_double(h);
+    const df ih = df_split(ihd), ih2 = df_split(ihd * ihd);
 
     // moments of the h-scaled design rows (the self row adds 1 to the count)
     df M[15], Z[6];
@@ -557,39 +568,49 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
     for (int p = 0; p < 6; p++)
 #pragma unroll
         for (int q = 0; q <= p; q++) G[tri(p, q)] = M[moment_index(mono_a(p) + mono_a(q), mono_b(p) + mono_b(q))];
-    float L[21];
-    if (!chol6(G, L) || !(cond1_6(G, L) <= kCondCap)) return false;
+    float L[21], il[6];
+    if (!chol6(G, L, il) || !(cond1_6(G, L, il) <= kCondCap)) return false;
 
-    // surface fit a~ = G^-1 V^T zeta, then the metric and A_1..A_5 at the origin
-    df at[6];
-    if (!solve6_refined(G, L, Z, at)) return false;
-    const df one = df_make(1.0f);
-    const df zx = at[1], zy = at[2];
-    const df zxx = df_mul(df_mul_f(at[3], 2.0f), ih), zxy = df_mul(at[4], ih),
-             zyy = df_mul(df_mul_f(at[5], 2.0f), ih);
-    const df zx2 = df_mul(zx, zx), zy2 = df_mul(zy, zy);
-    const df iW = df_div(one, df_add(one, df_add(zx2, zy2)));
-    const df g11 = df_mul(df_add(one, zy2), iW), g12 = df_neg(df_mul(df_mul(zx, zy), iW));
-    const df g22 = df_mul(df_add(one, zx2), iW);
-    const df Hs = df_add(df_add(df_mul(g11, zxx), df_mul_f(df_mul(g12, zxy), 2.0f)), df_mul(g22, zyy));
-    const df A1 = df_neg(df_mul(df_mul(Hs, zx), iW)), A2 = df_neg(df_mul(df_mul(Hs, zy), iW));
-    // the least-squares comparator drops the centre-value term (c~_0 = 0, no self correction)
-    const df c0 = A.variant == MVGD_ROW_LS ? df_make(0.f) : df_mul_f(df_add(g11, g22), 2.0f);
-    const df ct[6] = {c0, df_mul(A1, h), df_mul(A2, h), df_mul_f(g11, 2.0f), df_mul_f(g12, 2.0f),
-                      df_mul_f(g22, 2.0f)};
-
-    // g = G^-1 c~; the row is y = V g scaled by 1/h^2, with the self correction
-    df g[6];
-    if (!solve6_refined(G, L, ct, g)) return false;
-    const df ih2 = df_mul(ih, ih);
+    // surface fit a~ = G^-1 V^T zeta, then the metric and A_1..A_5 at the origin, then
+    // g = G^-1 c~ (the row is y = V g scaled by 1/h^2, with the self correction): one
+    // body for both solves, the kernel's code is past what the instruction cache holds
+    df g[6], rhs[6], c0 = df_make(0.f);
+#pragma unroll
+    for (int q = 0; q < 6; q++) rhs[q] = Z[q];
+#pragma unroll 1
+    for (int pass = 0; pass < 2; pass++) {
+        if (!solve6_refined(G, L, il, rhs, g)) return false;
+        if (pass == 1) break;
+        const df one = df_make(1.0f);
+        const df zx = g[1], zy = g[2];
+        const df zxx = df_mul(df_mul_f(g[3], 2.0f), ih), zxy = df_mul(g[4], ih),
+                 zyy = df_mul(df_mul_f(g[5], 2.0f), ih);
+        const df zx2 = df_mul(zx, zx), zy2 = df_mul(zy, zy);
+        const df iW = df_div(one, df_add(one, df_add(zx2, zy2)));
+        const df g11 = df_mul(df_add(one, zy2), iW), g12 = df_neg(df_mul(df_mul(zx, zy), iW));
+        const df g22 = df_mul(df_add(one, zx2), iW);
+        const df Hs = df_add(df_add(df_mul(g11, zxx), df_mul_f(df_mul(g12, zxy), 2.0f)), df_mul(g22, zyy));
+        const df A1 = df_neg(df_mul(df_mul(Hs, zx), iW)), A2 = df_neg(df_mul(df_mul(Hs, zy), iW));
+        // the least-squares comparator drops the centre-value term (c~_0 = 0, no self correction)
+        if (A.variant != MVGD_ROW_LS) c0 = df_mul_f(df_add(g11, g22), 2.0f);
+        rhs[0] = c0;
+        rhs[1] = df_mul(A1, h);
+        rhs[2] = df_mul(A2, h);
+        rhs[3] = df_mul_f(g11, 2.0f);
+        rhs[4] = df_mul_f(g12, 2.0f);
+        rhs[5] = df_mul_f(g22, 2.0f);
+    }
     const df w0 = df_mul(df_sub(g[0], c0), ih2);
     bool finite = df_isfinite(w0);
     for (int s = 0; s < k; s++) {
         const df xi = {MF(s, 0), MF(s, 1)}, eta = {MF(s, 2), MF(s, 3)};
-        df y = df_add(g[0], df_add(df_mul(xi, g[1]), df_mul(eta, g[2])));
-        y = df_add(y, df_add(df_mul(df_mul(xi, xi), g[3]),
-                             df_add(df_mul(df_mul(xi, eta), g[4]), df_mul(df_mul(eta, eta), g[5]))));
-        const df w = df_mul(y, ih2);
+        df_acc ax = acc_from(g[1]), ae = acc_from(g[2]), y = acc_from(g[0]);
+        acc_fma(ax, xi, g[3]);
+        acc_fma(ax, eta, g[4]);
+        acc_fma(ae, eta, g[5]);
+        acc_fma(y, xi, acc_value(ax));
+        acc_fma(y, eta, acc_value(ae));
+        const df w = df_mul(acc_value(y), ih2);
         finite = finite && df_isfinite(w);
         MF(s, 4) = w.hi;
         MF(s, 5) = w.lo;
