@@ -109,30 +109,18 @@ struct CtlLayout {
     unsigned* bar;
     int* words;     // err, active, nrestart, stop
     const Prob** prob;
-    int* chunk_req[kAmgMaxLevels + 1];   // [0] fine, [l] level l, [kAmgMaxLevels] coarsest
-    int* chunk_base[kAmgMaxLevels + 1];
+    int* chunk_base[kAmgMaxLevels + 1];  // [0] fine, [l] level l, [kAmgMaxLevels] coarsest
     size_t bytes;
 };
 
-constexpr int kCoarseUnits = (kAmgCoarsest + kThreads / kWarp - 1) / (kThreads / kWarp);
-
-CtlLayout ctl_layout(void* ws, int max_req, int64_t max_chunks) {
+CtlLayout ctl_layout(void* ws, int max_req) {
     CtlLayout C;
     memset(&C, 0, sizeof(C));
     Carver cv(ws);
     C.bar = cv.take<unsigned>(2);
     C.words = cv.take<int>(4);
     C.prob = cv.take<const Prob*>(max_req);
-    for (int t = 0; t <= kAmgMaxLevels; t++) {
-        // level l >= 1 of a request has n_l <= n / 8^l + 1 rows in ceil(n_l G / kThreads)
-        // <= n_l / 8 + 1 units (G <= 32): over all requests at most
-        // total_rows / 8^(l+1) + 2 count (one more per request kept as margin), and
-        // total_rows <= kCh max_chunks
-        const int64_t units = t == kAmgMaxLevels ? (int64_t)max_req * kCoarseUnits
-                              : (t == 0 ? max_chunks : ((int64_t)kCh * max_chunks >> (3 * (t + 1))) + 3 * max_req);
-        C.chunk_req[t] = cv.take<int>(units);
-        C.chunk_base[t] = cv.take<int>(max_req);
-    }
+    for (int t = 0; t <= kAmgMaxLevels; t++) C.chunk_base[t] = cv.take<int>(max_req + 1);
     C.bytes = cv.used;
     return C;
 }
@@ -231,20 +219,18 @@ struct TableArgs {
 
 // Request and chunk tables from by-value parameters (capturable in a graph);
 // the first group also resets the barrier and the control words.
-__global__ void k_build_table(TableArgs A, int base, const Prob** prob, int* chunk_req, int* chunk_base,
-                              unsigned* bar, int* words, int first_group) {
+__global__ void k_build_table(TableArgs A, int base, const Prob** prob, int* chunk_base, unsigned* bar,
+                              int* words, int first_group) {
     __shared__ int start[kTableMax + 1];
     if (threadIdx.x == 0) {
         start[0] = A.first_chunk;
         for (int i = 0; i < A.count; i++) start[i + 1] = start[i] + A.nchunk[i];
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < A.count; i += blockDim.x) {
-        if (prob) prob[base + i] = A.prob[i];
+    for (int i = threadIdx.x; i <= A.count; i += blockDim.x) {
+        if (prob && i < A.count) prob[base + i] = A.prob[i];
         chunk_base[base + i] = start[i];
     }
-    for (int i = 0; i < A.count; i++)
-        for (int c = start[i] + threadIdx.x; c < start[i + 1]; c += blockDim.x) chunk_req[c] = base + i;
     if (first_group && threadIdx.x == 0) {
         bar[0] = 0;
         bar[1] = 0;
@@ -254,7 +240,7 @@ __global__ void k_build_table(TableArgs A, int base, const Prob** prob, int* chu
 }
 
 // The tables, control words and counts of a launch of one request: it needs no
-// unit tables (see unit_req).
+// unit tables (its units are numbered from 0).
 __global__ void k_start_one(const Prob* req, const Prob** prob, unsigned* bar, int* words) {
     if (threadIdx.x != 0) return;
     prob[0] = req;
@@ -323,8 +309,6 @@ int gather_blocks(int64_t elems) {
     int64_t gb = (elems + 255) / 256;
     return (int)(gb > 8192 ? 8192 : (gb < 1 ? 1 : gb));
 }
-
-int64_t max_chunks_for(int count, int64_t total_rows) { return total_rows / kCh + count + 1; }
 
 }  // namespace
 }  // namespace mvgd
@@ -417,7 +401,7 @@ MVGD_API mvgd_status mvgd_request_init(void* req_ws, size_t req_bytes, const mvg
 
 MVGD_API size_t mvgd_iterate_workspace_bytes(int32_t max_requests, int64_t max_total_rows) {
     if (max_requests < 1 || max_total_rows < 1) return 0;
-    return ctl_layout(nullptr, max_requests, max_chunks_for(max_requests, max_total_rows)).bytes;
+    return ctl_layout(nullptr, max_requests).bytes;
 }
 
 MVGD_API mvgd_status mvgd_iterate(const mvgd_request* reqs, int32_t count, int32_t prec, int32_t precond,
@@ -447,7 +431,7 @@ MVGD_API mvgd_status mvgd_iterate(const mvgd_request* reqs, int32_t count, int32
     if (ctl_bytes < mvgd_iterate_workspace_bytes(count, total_rows)) return MVGD_EWORKSPACE;
     if (max_iterations == 0) return MVGD_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    CtlLayout C = ctl_layout(ctl_ws, count, max_chunks_for(count, total_rows));
+    CtlLayout C = ctl_layout(ctl_ws, count);
     ReqTable tab;
     memset(&tab, 0, sizeof(tab));
     tab.prob = C.prob;
@@ -479,7 +463,10 @@ MVGD_API mvgd_status mvgd_iterate(const mvgd_request* reqs, int32_t count, int32
         while (g > 1 && rows * g > threads) g >>= 1;
         tab.G[l] = g;
     }
-    tab.local = count == 1 && (reqs[0].n + kCh - 1) / kCh <= kFinWarpTiles && (amg || !mixed);
+    tab.sharing = count > 1 ? S_LISTED
+                            : ((reqs[0].n + kCh - 1) / kCh <= kFinWarpTiles && (amg || !mixed) ? S_LOCAL : S_SINGLE);
+    tab.ntab = amg ? (mlev > 0 ? mlev + 1 : 2) : 1;
+    tab.act = count > 1 && act_bytes(count, tab.ntab) <= kActBytes;
     // rows of the coarsest level a block takes: eight (a warp each), fewer while the
     // blocks of one request last -- the FP64 sums of eight warps queue for one SM's pipe
     tab.coarse_rows = kThreads / kWarp;
@@ -516,11 +503,10 @@ MVGD_API mvgd_status mvgd_iterate(const mvgd_request* reqs, int32_t count, int32
                 units += A.nchunk[i];
             }
             if (count > 1)
-                k_build_table<<<1, 256, 0, s>>>(A, g, t == 0 ? C.prob : nullptr, C.chunk_req[t], C.chunk_base[t],
-                                                C.bar, C.words, t == 0 && g == 0);
+                k_build_table<<<1, 256, 0, s>>>(A, g, t == 0 ? C.prob : nullptr, C.chunk_base[t], C.bar, C.words,
+                                                t == 0 && g == 0);
         }
         ChunkTable& T = coarse ? tab.coarse : (t == 0 ? tab.fine : tab.lvl[t]);
-        T.chunk_req = C.chunk_req[t];
         T.chunk_base = C.chunk_base[t];
         T.nchunks = units;
     }

@@ -863,12 +863,17 @@ __device__ void advance(const Prob& P, int ph, RhsState& T, const double* c, con
     }
 }
 
-// Work units of one kind of step: unit c belongs to request chunk_req[c] and
-// is its unit c - chunk_base[request].
+// Work units of one kind of step: request i's are chunk_base[i] .. chunk_base[i + 1] - 1.
 struct ChunkTable {
-    const int* chunk_req;   // [nchunks]
-    const int* chunk_base;  // [count]
+    const int* chunk_base;  // [count + 1] (several requests)
     int nchunks, pad;
+};
+
+// How a launch's blocks find their units.
+enum Sharing : int {
+    S_SINGLE = 0,  // one request: every gridDim-th unit
+    S_LOCAL = 1,   // the same, with few tiles: every block keeps the states itself (local_advance)
+    S_LISTED = 2   // several requests: a run of the running ones' units (Units)
 };
 
 // A launch of one request may cut its right-hand sides into `groups` of `gq`
@@ -884,7 +889,9 @@ struct ReqTable {
     int mlev;                      // largest (levels - 1) among the requests
     int nreq;                      // requests in the launch (1: every unit is request 0's, no lookups)
     int groups, gq;                // right-hand-side groups (1 with several requests)
-    int local;                     // every block keeps the states itself (see local_advance)
+    int sharing;                   // Sharing
+    int act;                       // S_LISTED: the list of running requests is kept
+    int ntab;                      // tables in use: fine, lvl[1 .. ntab-2] and coarse
     int coarse_rows;               // rows of a coarsest-level unit (a warp each, at most 8)
     int G[kAmgMaxLevels];          // [l], l >= 1: amg_group of the launch's rows at level l (see amg_lanes)
 };
@@ -897,15 +904,30 @@ __device__ __forceinline__ int block_count(const ReqTable& tab) {
     return tab.groups == 1 ? (int)gridDim.x : (int)gridDim.x / tab.groups;
 }
 
-// Request of unit c of table T, and the unit's place in that request.
-template <bool LOCAL>
-__device__ __forceinline__ int unit_req(const ReqTable& tab, const ChunkTable& T, int c) {
-    return LOCAL || tab.nreq == 1 ? 0 : T.chunk_req[c];
-}
-template <bool LOCAL>
-__device__ __forceinline__ int unit_place(const ReqTable& tab, const ChunkTable& T, int ri, int c) {
-    return LOCAL || tab.nreq == 1 ? c : c - T.chunk_base[ri];
-}
+// Several requests (S_LISTED).  A block that takes every gridDim-th unit of a step
+// meets another request at almost every unit, and each change costs a descriptor and
+// state load and, in reducing steps, an arrival: 4 us and more a tile with 32 clouds.
+// A run of consecutive units meets one or two requests.  But requests finish at
+// different times, and a fixed run of a finished request's units would leave its block
+// idle.  So the blocks keep the list of running requests in shared memory, with the
+// prefix of their unit counts per table, and cut the running units into equal runs;
+// the list is formed anew when the launch's count of running right-hand sides changes.
+// Two steps keep the stride, for a run of the dearest request's units would hold up the
+// rest: the coarsest solves (a row costs its request's nc) and an A with restarts in it
+// (a restart's FP64 residual is several inner steps): 48 -> 38 and 168 -> 116 us.
+//   act[j]: running request j;  pre[t][j]: running units of table t before it (pre[t][na]:
+//   all of them).
+// Where that would take more than kActBytes (some 400 requests) the runs are cut from
+// all requests' units, finished or not, by the tables themselves.
+__host__ __device__ constexpr size_t act_bytes(int count, int ntab) { return sizeof(int) * (size_t)(count + 1) * (1 + ntab); }
+constexpr size_t kActBytes = 8 << 10;
+
+// A block's units of one step.
+struct Units {
+    int lo, step, cnt;  // units lo, lo + step, ... (cnt of them; S_LISTED: of the running ones)
+    int cur;            // S_LISTED: place in the list of the unit taken last
+    const int* pre;     // S_LISTED: the list's unit counts
+};
 
 // The sums of a step's tile partials (nch channels) of a request of few tiles, into
 // tot[channel * QT + q]: a warp an entry, tiles across its lanes.  Block-wide.
@@ -1056,24 +1078,21 @@ __device__ __forceinline__ void arrive_and_finalize(const Prob& P, int ph, int s
 
 enum VStep : int { V_DOWN = 0, V_COARSE = 1, V_UP = 2 };
 
-// The tile this block takes after tile c in a step over table T, if it is
-// request ri's and this warp's slice of it holds rows (its slice in *slice2);
-// else -1.  Such a tile is staged exactly like tile c, so its slice can be
-// requested ahead.
-template <bool LOCAL>
-__device__ __forceinline__ int next_tile(const ReqTable& tab, const ChunkTable& T, int c, int nblk, int ri,
-                                         int64_t nrows, int wid, int64_t& slice2) {
-    const int c2 = c + nblk;
-    if (c2 < 0 || c2 >= T.nchunks || unit_req<LOCAL>(tab, T, c2) != ri) return -1;
-    slice2 = (int64_t)unit_place<LOCAL>(tab, T, ri, c2) * (kCh / kSlice) + wid;
+// The tile a block takes after tile c of a request of nrows rows, if this warp's
+// slice of it holds rows (its slice in *slice2); else -1.  Such a tile is staged
+// exactly like tile c, so its slice can be requested ahead.
+__device__ __forceinline__ int next_tile(int c, int step, int nchunks, int64_t nrows, int wid, int64_t& slice2) {
+    const int c2 = c + step;
+    if (c2 < 0 || c2 >= nchunks) return -1;
+    slice2 = (int64_t)c2 * (kCh / kSlice) + wid;
     return slice2 * kSlice < nrows ? c2 : -1;
 }
 
-// LOCAL: one request of few tiles, every block keeps the states itself (local_advance).
-template <bool MIXED, int QT, bool AMG, bool LOCAL>
+template <bool MIXED, int QT, bool AMG, int SHARING>
 __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     k_solve(ReqTable tab, Ctl ctl, int iter_budget, int kmax, int nbuf) {
     using VT = typename std::conditional<MIXED, float, double>::type;
+    constexpr bool LOCAL = SHARING == S_LOCAL, listed = SHARING == S_LISTED;
     __shared__ RhsState S[QT];
     __shared__ __align__(16) Prob sP;
     __shared__ __align__(16) AmgHeader sH;
@@ -1106,6 +1125,11 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     }
     __syncthreads();
 
+    extern __shared__ __align__(16) unsigned char stage_smem[];
+    int* const act = reinterpret_cast<int*>(stage_smem + (size_t)nbuf * (kThreads / kWarp) * stage_bytes_per_warp<VT>(kmax));
+    __shared__ int act_sum[kThreads / kWarp];
+    int nact = 0;  // running requests in the list
+    bool uneven = false;  // some right-hand side restarts in this iteration's A
     bool inner[QT], restart[QT];
     bool any_inner = false, any_restart = false, all_done = true;
     float c1[QT], c2[QT];
@@ -1202,7 +1226,103 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     // backwards in turn, so that the slice a warp holds from one step is the first of
     // the next: a block of 1M rows' nine tiles reads eight (an iteration 389 -> 382 us).
     int rev = 0;
-    auto unit_count = [&](const ChunkTable& T) { return bid < T.nchunks ? (T.nchunks - 1 - bid) / nblk + 1 : 0; };
+    auto table = [&](int t) -> const ChunkTable& { return t == 0 ? tab.fine : (t == tab.ntab - 1 ? tab.coarse : tab.lvl[t]); };
+    // The list of running requests and the prefixes of their units (block-wide).
+    auto relist = [&]() {
+        const int count = tab.nreq, pitch = count + 1;
+        if (!tab.act) {
+            nact = count;
+            return;
+        }
+        __syncthreads();
+        nact = 0;
+        st.have = -1;  // tiles are renumbered
+        for (int i0 = 0; i0 < count; i0 += kThreads) {
+            const int i = i0 + tid;
+            bool on = false;
+            if (i < count) {
+                const Prob* R = tab.prob[i];
+                const RhsState* rs = R->st;
+                for (int q = 0; q < R->Q; q++) on |= __ldcg(&rs[q].mode) != M_DONE;
+            }
+            const unsigned who = __ballot_sync(0xffffffffu, on);
+            if (lane == 0) act_sum[wid] = __popc(who);
+            __syncthreads();
+            int at = nact, all = 0;
+            for (int w = 0; w < kThreads / kWarp; w++) {
+                if (w < wid) at += act_sum[w];
+                all += act_sum[w];
+            }
+            if (on) act[at + __popc(who & ((1u << lane) - 1u))] = i;
+            nact += all;
+            __syncthreads();
+        }
+        for (int t = wid; t < tab.ntab; t += kThreads / kWarp) {
+            const ChunkTable& T = table(t);
+            int* pre = act + pitch * (1 + t);
+            int run = 0;
+            for (int j0 = 0; j0 < nact; j0 += 32) {
+                const int j = j0 + lane;
+                const int n = j < nact ? T.chunk_base[act[j] + 1] - T.chunk_base[act[j]] : 0;
+                int x = n;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, x, o);
+                    if (lane >= o) x += y;
+                }
+                if (j < nact) pre[j] = run + x - n;
+                run += __shfl_sync(0xffffffffu, x, 31);
+            }
+            if (lane == 0) pre[nact] = run;
+        }
+        __syncthreads();
+    };
+    // This block's units of table t; unit i of them: its request, its place in the
+    // request, and (returned) its number among the units in the list.
+    // runs: a run of them (S_LISTED), else every nblk-th.
+    auto units_of = [&](int t, bool runs) {
+        Units U;
+        U.cur = 0;
+        if (listed) {
+            U.pre = tab.act ? act + (tab.nreq + 1) * (1 + t) : table(t).chunk_base;
+            const int n = U.pre[nact];
+            if (runs) {
+                U.lo = (int)(bid * (int64_t)n / nblk);
+                U.cnt = (int)((bid + 1) * (int64_t)n / nblk) - U.lo;
+                U.step = 1;
+            } else {
+                U.lo = bid;
+                U.cnt = bid < n ? (n - 1 - bid) / nblk + 1 : 0;
+                U.step = nblk;
+            }
+            int hi = nact;  // the last j with pre[j] <= lo
+            while (hi - U.cur > 1) {
+                const int mid = (U.cur + hi) >> 1;
+                if (U.pre[mid] <= U.lo) U.cur = mid;
+                else hi = mid;
+            }
+        } else {
+            const int n = table(t).nchunks;
+            U.pre = nullptr;
+            U.lo = bid;
+            U.step = nblk;
+            U.cnt = bid < n ? (n - 1 - bid) / nblk + 1 : 0;
+        }
+        return U;
+    };
+    auto unit_at = [&](Units& U, int i, int& ri, int& place) -> int {
+        if (listed) {
+            const int a = U.lo + i * U.step;
+            while (a >= U.pre[U.cur + 1]) U.cur++;
+            while (a < U.pre[U.cur]) U.cur--;
+            ri = tab.act ? act[U.cur] : U.cur;
+            place = a - U.pre[U.cur];
+            return a;
+        }
+        ri = 0;
+        place = U.lo + i * nblk;
+        return place;
+    };
 
     // One request of few tiles (LOCAL): after a reducing step's barrier every block
     // sums the tile partials and advances its own copy of the states, the same
@@ -1255,10 +1375,10 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
             __syncthreads();
             nred = 0;
         };
-        const int cnt = unit_count(tab.fine);
+        Units U = units_of(0, !(ph == P_A && uneven));
         for (int i = 0;; i++) {
-            const int c = bid + (rev ? cnt - 1 - i : i) * nblk;
-            const int ri = i < cnt ? unit_req<LOCAL>(tab, tab.fine, c) : -1;
+            int ri = -1, lc = 0, c = 0;
+            if (i < U.cnt) c = unit_at(U, rev ? U.cnt - 1 - i : i, ri, lc);
             if (ri != cur || ri < 0) {  // (a block may have no level-0 tile at all)
                 // leaving request `cur`: publish this block's tiles of it
                 if (cur >= 0 && reduce && tiles > 0) {
@@ -1274,7 +1394,6 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
             }
             if (all_done) continue;  // the whole request is finished: no work, no arrival
             const Prob& P = sP;
-            const int lc = unit_place<LOCAL>(tab, tab.fine, ri, c);
             const int64_t r = (int64_t)lc * kCh + tid;
             const int64_t slice = (int64_t)lc * (kCh / kSlice) + wid;
             F2 af[NC][QT];
@@ -1287,7 +1406,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
             const bool staged = (ph == P_A || ph == P_B) && any_inner && slice * kSlice < P.n && st.ok();
             if (staged) {
                 int64_t slice2 = 0;
-                const int cn = next_tile<LOCAL>(tab, tab.fine, c, rev ? -nblk : nblk, ri, P.n, wid, slice2);
+                const int cn = listed ? -1 : next_tile(c, rev ? -nblk : nblk, tab.fine.nchunks, P.n, wid, slice2);
                 // FP32 multigrid flow: the hierarchy's level-0 weights (the operator's hi
                 // values, copied at set-up), the array the V-cycle's level-0 steps read too
                 const void* vsrc = (AMG && MIXED) ? static_cast<const void*>(P.amg->lv[0].val) : P.val;
@@ -1355,17 +1474,20 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     // x into u).  The rows and their arithmetic are those of fine_phase.
     auto pre_phase = [&](int ph) -> bool {
         constexpr int NT = MIXED ? (QT == 1 ? 4 : 2) : (QT == 1 ? 2 : 1);  // operands in registers
-        const int G = nblk;
-        for (int c = bid; c < tab.fine.nchunks;) {
-            const int ri = unit_req<LOCAL>(tab, tab.fine, c);
+        const int step = listed ? 1 : nblk;  // from a unit's place to the block's next one's
+        Units U = units_of(0, true);
+        for (int i = 0; i < U.cnt;) {
+            int ri, lc;
+            unit_at(U, i, ri, lc);
             if (ri != held) enter(ri, ph);
-            int n = 1;
-            while (n < NT && c + n * G < tab.fine.nchunks && unit_req<LOCAL>(tab, tab.fine, c + n * G) == ri) n++;
+            int n;
+            if (listed) n = min(NT, min(U.cnt - i, U.pre[U.cur + 1] - U.lo - i));
+            else n = min(NT, U.cnt - i);
             if (!all_done) {
                 const Prob& P = sP;
                 if (any_restart) {
                     for (int k = 0; k < n; k++) {
-                        const int64_t r = (int64_t)unit_place<LOCAL>(tab, tab.fine, ri, c + k * G) * kCh + tid;
+                        const int64_t r = (int64_t)(lc + k * step) * kCh + tid;
                         if (r < P.n) amg_pre_row<MIXED, QT>(P, r, ph, S, inner, restart);
                     }
                 } else {
@@ -1373,13 +1495,13 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
                     bool ok[NT];
 #pragma unroll
                     for (int k = 0; k < NT; k++) {
-                        rows[k] = (int64_t)unit_place<LOCAL>(tab, tab.fine, ri, c + k * G) * kCh + tid;
+                        rows[k] = (int64_t)(lc + k * step) * kCh + tid;
                         ok[k] = k < n && rows[k] < P.n;
                     }
                     amg_pre_rows<MIXED, QT, NT>(P, rows, ok, ph, S, inner);
                 }
             }
-            c += n * G;
+            i += n;
         }
         const bool ok = grid_sync(ctl.bar, bar_epoch, ctl.err, ctl.limit,
                                   !(ctl.withhold && blockIdx.x == 0 && bar_epoch == 0));
@@ -1390,12 +1512,11 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     // One step of the V-cycle applied to p (side 0) or s (side 1) of every
     // INNER right-hand side, then the grid barrier.
     auto vstep = [&](int kind, int l, int side) -> bool {
-        const ChunkTable& T = kind == V_COARSE ? tab.coarse : (l == 0 ? tab.fine : tab.lvl[l]);
         int cur = -1;
-        const int cnt = unit_count(T);
-        for (int i = 0; i < cnt; i++) {
-            const int c = bid + (rev && kind != V_COARSE && l == 0 ? cnt - 1 - i : i) * nblk;
-            const int ri = unit_req<LOCAL>(tab, T, c);
+        Units U = kind == V_COARSE ? units_of(tab.ntab - 1, false) : units_of(l, true);
+        for (int i = 0; i < U.cnt; i++) {
+            int ri, lc;
+            const int c = unit_at(U, rev && kind != V_COARSE && l == 0 ? U.cnt - 1 - i : i, ri, lc);
             if (ri != cur) {
                 cur = ri;
                 // V-cycle steps leave the states alone: the one loaded by the
@@ -1407,7 +1528,6 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
             if (!any_inner || (kind != V_COARSE && l >= m)) continue;
             const AmgHeader& H = *P.amg;
             const int Q = P.Q;
-            const int lc = unit_place<LOCAL>(tab, T, ri, c);
             const VT* B0 = static_cast<const VT*>(side == 0 ? P.p[0] : P.s);
             VT* X0 = static_cast<VT*>(side == 0 ? P.ph : P.sh);
             if (kind == V_COARSE) {
@@ -1440,7 +1560,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
                 if (!st.ok()) continue;
                 const int64_t slice = (int64_t)lc * (kCh / kSlice) + wid;
                 int64_t slice2 = 0;
-                const int cn = next_tile<LOCAL>(tab, tab.fine, c, rev ? -nblk : nblk, ri, nl, wid, slice2);
+                const int cn = listed ? -1 : next_tile(c, rev ? -nblk : nblk, tab.fine.nchunks, nl, wid, slice2);
                 b = st.acquire(kmax, nbuf, MVGD_STAGE_BAR, c, slice, cn, slice2, P.col, H.lv[0].val, 4, P.k, ctl.err);
                 colS = st.col(kmax, nbuf, b);
                 w0S = static_cast<const float*>(st.val(kmax, nbuf, b));
@@ -1536,8 +1656,14 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     // the counts are stable between the barrier that follows their last change and the
     // next reducing step: identical in every block
     auto finished = [&]() { return *(volatile int*)ctl.active == 0 || *(volatile int*)ctl.stop != 0; };
+    int running = -1;  // the launch's running right-hand sides when the list was formed
     for (int it = 0; it < iter_budget; ++it) {
         bool ok = true, leave = false;
+        if (listed && *(volatile int*)ctl.active != running) {
+            running = *(volatile int*)ctl.active;
+            relist();
+        }
+        if (listed) uneven = *(volatile int*)ctl.nrestart > 0;
         if (AMG) {
             if constexpr (QT <= 2) {
                 ok = pre_phase(P_PRE_A);
@@ -1582,11 +1708,11 @@ int stage_buffers(int kmax) {
 }
 
 // Resident blocks of one instantiation (0: a CUDA error).
-template <bool MIXED, int QT, bool AMG, bool LOCAL>
-int solve_capacity(int kmax, size_t* smem_out = nullptr) {
+template <bool MIXED, int QT, bool AMG, int SHARING>
+int solve_capacity(int kmax, size_t* smem_out = nullptr, size_t more = 0) {
     using VT = typename std::conditional<MIXED, float, double>::type;
-    auto fn = k_solve<MIXED, QT, AMG, LOCAL>;
-    const size_t smem = stage_bytes_per_warp<VT>(kmax) * (kThreads / kWarp) * stage_buffers<VT>(kmax);
+    auto fn = k_solve<MIXED, QT, AMG, SHARING>;
+    const size_t smem = stage_bytes_per_warp<VT>(kmax) * (kThreads / kWarp) * stage_buffers<VT>(kmax) + more;
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -1599,11 +1725,12 @@ int solve_capacity(int kmax, size_t* smem_out = nullptr) {
     return sms * per_sm;
 }
 
-template <bool MIXED, int QT, bool AMG, bool LOCAL>
+template <bool MIXED, int QT, bool AMG, int SHARING>
 mvgd_status launch_solve_as(const ReqTable& tab, Ctl ctl, int budget, int kmax, cudaStream_t s) {
     using VT = typename std::conditional<MIXED, float, double>::type;
     size_t smem = 0;
-    int grid = solve_capacity<MIXED, QT, AMG, LOCAL>(kmax, &smem);
+    int grid = solve_capacity<MIXED, QT, AMG, SHARING>(
+        kmax, &smem, tab.act ? act_bytes(tab.nreq, tab.ntab) : 0);
     if (grid < 1) return MVGD_ECUDA;
     // a block for every unit of the step that has most of them (a level whose rows
     // must take many lanes, or the coarsest one of a small system, can have more
@@ -1619,7 +1746,7 @@ mvgd_status launch_solve_as(const ReqTable& tab, Ctl ctl, int budget, int kmax, 
     int nbuf = stage_buffers<VT>(kmax);
     ReqTable t = tab;
     void* args[] = {(void*)&t, (void*)&ctl, (void*)&budget, (void*)&kmax, (void*)&nbuf};
-    MVGD_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_solve<MIXED, QT, AMG, LOCAL>, dim3(grid), dim3(kThreads), args,
+    MVGD_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_solve<MIXED, QT, AMG, SHARING>, dim3(grid), dim3(kThreads), args,
                                               smem, s));
     return MVGD_OK;
 }
@@ -1632,9 +1759,10 @@ constexpr bool has_local() { return AMG || !MIXED; }
 template <bool MIXED, int QT, bool AMG>
 mvgd_status launch_solve(const ReqTable& tab, Ctl ctl, int budget, int kmax, cudaStream_t s) {
     if constexpr (has_local<MIXED, AMG>()) {
-        if (tab.local) return launch_solve_as<MIXED, QT, AMG, true>(tab, ctl, budget, kmax, s);
+        if (tab.sharing == S_LOCAL) return launch_solve_as<MIXED, QT, AMG, S_LOCAL>(tab, ctl, budget, kmax, s);
     }
-    return launch_solve_as<MIXED, QT, AMG, false>(tab, ctl, budget, kmax, s);
+    if (tab.sharing == S_LISTED) return launch_solve_as<MIXED, QT, AMG, S_LISTED>(tab, ctl, budget, kmax, s);
+    return launch_solve_as<MIXED, QT, AMG, S_SINGLE>(tab, ctl, budget, kmax, s);
 }
 
 template <bool MIXED, bool AMG>
@@ -1655,10 +1783,11 @@ mvgd_status dispatch_q(int Q, const ReqTable& tab, Ctl ctl, int budget, int kmax
 // groups of two; 7,001 rows x 4 in FP32: 124 and 64.
 template <bool MIXED, bool AMG>
 int rhs_group(int Q, int tiles, int kmax) {
+    constexpr int kOneRequest = has_local<MIXED, AMG>() ? S_LOCAL : S_SINGLE;
     const int64_t t = tiles;
-    if (t * Q <= solve_capacity<MIXED, 1, AMG, has_local<MIXED, AMG>()>(kmax)) return 1;
-    if (Q > 2 && Q % 2 == 0 && t * (Q / 2) <= solve_capacity<MIXED, 2, AMG, has_local<MIXED, AMG>()>(kmax)) return 2;
-    if (Q > 4 && Q % 4 == 0 && t * (Q / 4) <= solve_capacity<MIXED, 4, AMG, has_local<MIXED, AMG>()>(kmax)) return 4;
+    if (t * Q <= solve_capacity<MIXED, 1, AMG, kOneRequest>(kmax)) return 1;
+    if (Q > 2 && Q % 2 == 0 && t * (Q / 2) <= solve_capacity<MIXED, 2, AMG, kOneRequest>(kmax)) return 2;
+    if (Q > 4 && Q % 4 == 0 && t * (Q / 4) <= solve_capacity<MIXED, 4, AMG, kOneRequest>(kmax)) return 4;
     return Q;
 }
 
