@@ -60,8 +60,9 @@ int32_t mvgd_version(void);
  * the lower index.  The result is exact: identical to a brute-force search.
  *
  * order (optional out, int32 [n]) receives a locality order of the points
- * (the cell order of the search grid); pass it to mvgd_assemble so that the
- * solver works on rows whose neighbours are close in memory.
+ * (one Z-order curve through the cube around the cloud, 21 bits an axis, ties
+ * by index); pass it to mvgd_assemble so that the solver works on rows whose
+ * neighbours are close in memory.
  *
  * cell_size > 0 fixes the edge of the search grid's cells; 0 picks one from
  * an estimate of the k-th neighbour distance, and a negative value picks
@@ -136,8 +137,8 @@ typedef enum {
  * fit by Householder QR).  MVGD_FP32_REFINE rows are formed on the FP32 pipe
  * unless rule.arith == 1: offsets p_j - p_i in FP64, then covariance and
  * h-scaled local coordinates in double-float (pairs of FP32 numbers, about 48
- * bits), the 3x3 eigenvectors
- * from an FP32 Jacobi polished by FP64 Jacobi sweeps, and the least-squares
+ * bits), the 3x3 eigenvectors from FP32 Jacobi sweeps finished in FP64 (as in
+ * the FP64 arithmetic for k >= 8), and the least-squares
  * fits through normal equations solved with an FP32 Cholesky factor and
  * refined from double-float residuals (for k >= 8: a fit over fewer points is
  * square or nearly so and always uses FP64); the hi + lo weights then agree with the
@@ -429,7 +430,7 @@ mvgd_status mvgd_solve(const mvgd_ell *L, int32_t nrhs, double sigma, const doub
  * Aggregation multigrid.  The paper solves its systems with algebraic
  * multigrid (Sec. 4.2, whose timing table grows about linearly in N)
  * without naming a variant.  Here: plain aggregation on the stored row order
- * (consecutive rows are spatial neighbours after the kNN step's cell sort).
+ * (consecutive rows are spatial neighbours in the kNN step's Z-order).
  *   - aggregate I of a level = its MVGD_AMG_AGG consecutive rows I*AGG ..;
  *   - next level = Galerkin product P^T A P, P piecewise constant (FP64 sums,
  *     kept as FP32 for the cycle);

@@ -24,7 +24,7 @@ import torch
 
 from . import _lib as LB
 from . import api
-from .serve import amg_setup_kernels
+from .serve import amg_setup_kernels, iterate_kernels, knn_kernels
 
 
 @dataclass
@@ -126,7 +126,7 @@ class BatchPipeline:
             marks[1].record(main)
         if self.precond == LB.PRECOND_AMG:
             # the hierarchies on the stream pool: each set-up is a chain of small
-            # launches (the coarsest inverse is one block), so clouds overlap
+            # launches (the coarsest inverse is one cluster), so clouds overlap
             built = torch.cuda.Event()
             built.record(main)
             for i, slot in enumerate(self.slots):
@@ -169,8 +169,8 @@ class BatchPipeline:
 
     @property
     def kernels_per_run(self) -> int:
-        per_cloud_knn = 11
-        return (len(self.slots) * (per_cloud_knn + 1 + 3 + 2)  # knn, inverse order, init (2 gathers+1), finish (2)
+        return (sum(knn_kernels(s.n) for s in self.slots)
+                + len(self.slots) * (1 + 3 + 2)                 # inverse order, init (2 gathers+1), finish (2)
                 + 1 + (len(self.slots) + 47) // 48              # batched assembly + descriptor uploads
-                + (len(self.slots) + 255) // 256 + 3            # iterate: tables, count, solver, exit marks
+                + iterate_kernels([s.n for s in self.slots], self.precond)
                 + (sum(amg_setup_kernels(s.n) for s in self.slots) if self.precond == LB.PRECOND_AMG else 0))

@@ -17,8 +17,11 @@
 // FP32 path forms them on the fly and saves two barriers.  Rows are cut into
 // fixed chunks of kCh rows; a chunk's partials are reduced in a fixed order
 // and the block that finishes a request's last chunk of a phase sums that
-// request's partials in chunk order and advances its per-RHS state.  Results
+// request's partials in chunk order and advances its per-RHS state (in a launch
+// of one request of few chunks every block does both, for itself).  Results
 // therefore depend neither on the grid size nor on the other requests.
+// The kernel is in solve_kernel.cuh; this file has the host side and the small
+// kernels around it.
 //
 // Per right-hand side:
 //   RESTART  FP64 true residual r64 = f - A u (FP32 path: on hi + lo weights,

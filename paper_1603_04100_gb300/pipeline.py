@@ -13,11 +13,11 @@ import torch
 
 from . import _lib as LB
 from . import api
+from .serve import amg_setup_kernels, knn_kernels
 
 # kernels each stage launches (the C ABI's own launches, not counting memsets/copies)
-KERNELS_KNN = 11          # bbox x2, occupancy, params, count, scan x3, scatter, bucket sort, query
 KERNELS_ASSEMBLE = 1      # + 1 inverse-order kernel with a locality order
-KERNELS_SOLVE = 9         # init: 2 gathers + state; iterate: table, count, solver, exit marks; finish: 2
+KERNELS_SOLVE = 8         # init: 2 gathers + state; iterate: start, solver, exit marks; finish: 2
 
 
 class Pipeline:
@@ -60,16 +60,11 @@ class Pipeline:
 
     @property
     def kernels_per_run(self) -> int:
-        k = KERNELS_KNN + KERNELS_ASSEMBLE + (1 if self.reorder else 0) + KERNELS_SOLVE
+        k = knn_kernels(self.n, self.reorder) + KERNELS_ASSEMBLE + (1 if self.reorder else 0) + KERNELS_SOLVE
         if self.precond == LB.PRECOND_ROWSCALE:
             k += 1                                   # row scaling
         if self.precond == LB.PRECOND_AMG:
-            lv = 1
-            m = self.n
-            while m > LB.AMG_COARSEST:
-                m = (m + LB.AMG_AGG - 1) // LB.AMG_AGG
-                lv += 1
-            k += 9 + 2 * (lv - 1)                    # hierarchy set-up (with the Newton-Schulz products)
+            k += amg_setup_kernels(self.n)
             k += (lv - 2 if lv > 2 else 0) + 1       # level and coarsest chunk tables
         return k
 

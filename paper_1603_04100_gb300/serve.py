@@ -86,9 +86,27 @@ def amg_levels(n: int) -> int:
 
 
 def amg_setup_kernels(n: int) -> int:
-    """Kernels mvgd_amg_setup launches: header, level 0, two per coarser level, dense, inverse, promotion
-    and four Newton-Schulz products."""
-    return 9 + 2 * (amg_levels(n) - 1)
+    """Kernels mvgd_amg_setup launches: header, level 0, one per coarser level, dense, inverse and four
+    Newton-Schulz products."""
+    return 8 + (amg_levels(n) - 1)
+
+
+def knn_kernels(n: int, order: bool = True) -> int:
+    """Kernels mvgd_knn launches: box, occupancy, count, two for the scan, scatter, query; the stored order in
+    one more block up to 8,192 points, else in eight radix passes of two."""
+    return 7 + (0 if not order else 1 if n <= 8192 else 16)
+
+
+def iterate_kernels(ns, precond: int) -> int:
+    """Kernels mvgd_iterate launches for requests of ns rows: solver and exit marks, and before them one kernel
+    for a single request; else the unit tables (fine; with multigrid levels 1 .. and the coarsest), 256 requests
+    a kernel, and the count of running right-hand sides."""
+    if len(ns) == 1:
+        return 3
+    tables = 1
+    if precond == LB.PRECOND_AMG:
+        tables += max(max(amg_levels(n) for n in ns) - 1, 1)
+    return tables * ((len(ns) + 255) // 256) + 3
 
 
 class Server:
@@ -149,7 +167,7 @@ class Server:
                 ws_knn = self.knn_ws[i % len(self.pool)]
                 LB.check("mvgd_knn", L.mvgd_knn(vp(pts), n, k, vp(nbr), vp(order), 0.0, vp(ws_knn), ws_knn.numel(),
                                                  api._stream(ps)))
-                self.launches += 11
+                self.launches += knn_kernels(n)
                 col, val, lo = api.ell_alloc(n, k, self.prec, self.device)
                 op = api.Operator(n, k, self.prec, col, val, lo, order)
                 ws = torch.empty(L.mvgd_request_workspace_bytes(n, k, q, self.prec, self.precond), dtype=torch.uint8,
@@ -210,11 +228,7 @@ class Server:
                                                      vp(self.ctl_ws), self.ctl_bytes, s))
             LB.check("mvgd_request_poll", L.mvgd_request_poll(reqs, cnt, vp(self.done_dev), s))
             self.done_host[:cnt].copy_(self.done_dev[:cnt], non_blocking=True)
-        groups = (cnt + 255) // 256
-        tables = 1
-        if self.precond == LB.PRECOND_AMG:
-            tables += max(amg_levels(x.req.n) - 1 for x in active)  # levels 1 .. mlev-1, and the coarsest
-        self.launches += groups * tables + 3 + groups              # tables, count, solver, exit marks, poll
+        self.launches += iterate_kernels([x.req.n for x in active], self.precond) + (cnt + 255) // 256  # + poll
         self.stream.synchronize()
         self.epochs += 1
         return [i for i in range(cnt) if int(self.done_host[i]) != 0]
