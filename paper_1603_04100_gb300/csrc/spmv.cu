@@ -34,10 +34,112 @@ __device__ __forceinline__ double ld_stream(const double* p) {
     return v;
 }
 
+// Row j of x (Q right-hand sides side by side), by the widest loads that Q allows: x is
+// 256-byte aligned (checked at the entry), so a row of an even Q starts on two elements'
+// boundary, one of Q = 4 or 8 on four's.  FP32, 1,048,576 rows, K = 20, eight vectors:
+// 213 -> 90 us (a warp's gather of one element of 32 rows takes as many L1 passes as one of
+// four); four of 100,003 rows, K = 16: 12.3 -> 10.3.
+template <int Q>
+__device__ __forceinline__ void load_x(const double* __restrict__ x, int64_t j, double (&v)[Q]) {
+    const double* p = x + j * Q;
+    if constexpr (Q % 2 == 0) {
+#pragma unroll
+        for (int q = 0; q < Q; q += 2) {
+            const double2 t = *reinterpret_cast<const double2*>(p + q);
+            v[q] = t.x;
+            v[q + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < Q; q++) v[q] = p[q];
+    }
+}
+template <int Q>
+__device__ __forceinline__ void load_x(const float* __restrict__ x, int64_t j, float (&v)[Q]) {
+    const float* p = x + j * Q;
+    if constexpr (Q % 4 == 0) {
+#pragma unroll
+        for (int q = 0; q < Q; q += 4) {
+            const float4 t = *reinterpret_cast<const float4*>(p + q);
+            v[q] = t.x;
+            v[q + 1] = t.y;
+            v[q + 2] = t.z;
+            v[q + 3] = t.w;
+        }
+    } else if constexpr (Q % 2 == 0) {
+#pragma unroll
+        for (int q = 0; q < Q; q += 2) {
+            const float2 t = *reinterpret_cast<const float2*>(p + q);
+            v[q] = t.x;
+            v[q + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < Q; q++) v[q] = p[q];
+    }
+}
+
+// Rows a block of the FP64 products.  With several right-hand sides they are bound by the
+// FP64 pipe (2 FMAs a clock an SM), and blocks of 256 leave some SMs a third more rows than
+// others (100,003 rows: 391 blocks on 152 SMs); one warp a block spreads them within 3 %
+// and a small operator over every SM.  A block of a warp also caps an SM at 32 warps, which
+// costs nothing where K is fixed at compile time and a row's loads are issued ahead, but does
+// with the loop over a K known at run time (524,288 rows, K = 30, one vector: 40 us with 256
+// threads, 45 with 32), which keeps 256.  The hi + lo product has two FP64 conversions and an
+// addition a weight more on that pipe and gains at every K (1,048,576 rows, K = 20:
+// 177 -> 172 us; 524,288, K = 31: 141 -> 131).
+constexpr int spmv_threads(int kk) { return kk > 0 ? 32 : 256; }
+constexpr int kHiloThreads = 32;
+
+// acc += the row's k slots in order, `weight(s)` times row col[s * kSlice] of x.  K fixed at
+// compile time: the columns, weights and rows of x of a batch are all requested before the
+// first product.  Else the compiler's unrolling, with wide loads of x only for eight vectors
+// (100,003 rows, K = 30, four: 32.7 us without, 33.4 with; 524,288 rows, eight: 277, 246).
+// In us, before (scalar loads, blocks of 256) -> now: 20,001 rows, K = 20, eight vectors
+// 25 -> 16; 524,288 rows, K = 24, eight 230 -> 197; 100,003 rows, K = 16, four 20.5 -> 20.0
+// (12 of them the FP64 pipe); 20,001 rows, K = 31, one 16 -> 6.2.
+template <int Q, int KK, typename Weight>
+__device__ __forceinline__ void add_slots(int k, const int32_t* __restrict__ col, const double* __restrict__ x,
+                                          double (&acc)[Q], Weight&& weight) {
+    constexpr int B = Q <= 2 ? 8 : 4;
+    int s0 = 0;
+    if constexpr (KK > 0) {
+#pragma unroll (KK / B)
+        for (; s0 + B <= KK; s0 += B) {
+            int32_t c[B];
+            double w[B], xj[B][Q];
+#pragma unroll
+            for (int u = 0; u < B; u++) c[u] = ld_stream(col + (int64_t)(s0 + u) * kSlice);
+#pragma unroll
+            for (int u = 0; u < B; u++) w[u] = weight(s0 + u);
+#pragma unroll
+            for (int u = 0; u < B; u++) load_x<Q>(x, c[u], xj[u]);
+#pragma unroll
+            for (int u = 0; u < B; u++)
+#pragma unroll
+                for (int q = 0; q < Q; q++) acc[q] = fma(w[u], xj[u][q], acc[q]);
+        }
+    }
+#pragma unroll 4
+    for (; s0 < k; s0++) {
+        const int64_t j = ld_stream(col + (int64_t)s0 * kSlice);
+        const double w = weight(s0);
+        double xj[Q];
+        if constexpr (KK > 0 || Q == 8) {
+            load_x<Q>(x, j, xj);
+        } else {
+#pragma unroll
+            for (int q = 0; q < Q; q++) xj[q] = x[j * Q + q];
+        }
+#pragma unroll
+        for (int q = 0; q < Q; q++) acc[q] = fma(w, xj[q], acc[q]);
+    }
+}
+
 // KK > 0: K fixed at compile time (every slot's loads can be issued at once);
 // KK == 0: K at run time.
 template <int Q, int KK>
-__global__ void __launch_bounds__(256) k_spmv_f64(int64_t n, int kr, const int32_t* __restrict__ col,
+__global__ void __launch_bounds__(spmv_threads(KK)) k_spmv_f64(int64_t n, int kr, const int32_t* __restrict__ col,
                                                    const double* __restrict__ val, double sigma, double alpha,
                                                    const double* __restrict__ x, double beta,
                                                    double* __restrict__ y) {
@@ -49,18 +151,12 @@ __global__ void __launch_bounds__(256) k_spmv_f64(int64_t n, int kr, const int32
     const int64_t cb = (r / kSlice) * (int64_t)(kSlice * k) + (r % kSlice);
     const double w0 = ld_stream(val + vb);
     double xi[Q], acc[Q];
+    load_x<Q>(x, r, xi);
 #pragma unroll
     for (int q = 0; q < Q; q++) {
-        xi[q] = x[r * Q + q];
         acc[q] = w0 * xi[q];
     }
-#pragma unroll (KK > 0 ? KK : 4)
-    for (int s = 0; s < k; s++) {
-        const int64_t j = ld_stream(col + cb + (int64_t)s * kSlice);
-        const double w = ld_stream(val + vb + (int64_t)(s + 1) * kSlice);
-#pragma unroll
-        for (int q = 0; q < Q; q++) acc[q] = fma(w, x[j * Q + q], acc[q]);
-    }
+    add_slots<Q, KK>(k, col + cb, x, acc, [&](int s) { return ld_stream(val + vb + (int64_t)(s + 1) * kSlice); });
 #pragma unroll
     for (int q = 0; q < Q; q++) {
         double out = alpha * (sigma * xi[q] - acc[q]);
@@ -81,17 +177,19 @@ __global__ void __launch_bounds__(256) k_spmv_f32(int64_t n, int kr, const int32
     const int64_t vb = (r / kSlice) * (int64_t)(kSlice * m) + (r % kSlice);
     const int64_t cb = (r / kSlice) * (int64_t)(kSlice * k) + (r % kSlice);
     float xi[Q], acc[Q];
+    load_x<Q>(x, r, xi);
 #pragma unroll
     for (int q = 0; q < Q; q++) {
-        xi[q] = x[r * Q + q];
         acc[q] = 0.0f;
     }
 #pragma unroll (KK > 0 ? KK : 4)
     for (int s = 0; s < k; s++) {
         const int64_t j = ld_stream(col + cb + (int64_t)s * kSlice);
         const float w = ld_stream(val + vb + (int64_t)(s + 1) * kSlice);
+        float xj[Q];
+        load_x<Q>(x, j, xj);
 #pragma unroll
-        for (int q = 0; q < Q; q++) acc[q] = fmaf(w, x[j * Q + q] - xi[q], acc[q]);
+        for (int q = 0; q < Q; q++) acc[q] = fmaf(w, xj[q] - xi[q], acc[q]);
     }
 #pragma unroll
     for (int q = 0; q < Q; q++) {
@@ -111,7 +209,7 @@ void launch_spmv_k(const mvgd_ell* L, int mode, double sigma, double alpha, cons
                                                  (float)alpha, static_cast<const float*>(x), (float)beta,
                                                  static_cast<float*>(y));
     else
-        k_spmv_f64<Q, KK><<<blocks, 256, 0, s>>>(n, L->k, L->col, static_cast<const double*>(L->val), sigma, alpha,
+        k_spmv_f64<Q, KK><<<(unsigned)((n + spmv_threads(KK) - 1) / spmv_threads(KK)), spmv_threads(KK), 0, s>>>(n, L->k, L->col, static_cast<const double*>(L->val), sigma, alpha,
                                                  static_cast<const double*>(x), beta, static_cast<double*>(y));
 }
 
@@ -119,12 +217,13 @@ template <int Q>
 mvgd_status launch_spmv(const mvgd_ell* L, int mode, double sigma, double alpha, const void* x, double beta,
                         void* y, cudaStream_t s) {
     if (mode == MVGD_SPMV_F32 || mode == MVGD_SPMV_F64) {
-        // the common K at compile time, any other at run time
+        // the common K and the largest at compile time, any other at run time
         switch (L->k) {
             case 12: launch_spmv_k<Q, 12>(L, mode, sigma, alpha, x, beta, y, s); break;
             case 16: launch_spmv_k<Q, 16>(L, mode, sigma, alpha, x, beta, y, s); break;
             case 20: launch_spmv_k<Q, 20>(L, mode, sigma, alpha, x, beta, y, s); break;
             case 24: launch_spmv_k<Q, 24>(L, mode, sigma, alpha, x, beta, y, s); break;
+            case 31: launch_spmv_k<Q, 31>(L, mode, sigma, alpha, x, beta, y, s); break;
             default: launch_spmv_k<Q, 0>(L, mode, sigma, alpha, x, beta, y, s); break;
         }
     } else {
@@ -135,7 +234,7 @@ mvgd_status launch_spmv(const mvgd_ell* L, int mode, double sigma, double alpha,
 }
 
 template <int Q>
-__global__ void __launch_bounds__(256) k_spmv_hilo(int64_t n, int k, const int32_t* __restrict__ col,
+__global__ void __launch_bounds__(kHiloThreads) k_spmv_hilo(int64_t n, int k, const int32_t* __restrict__ col,
                                                     const float* __restrict__ hi, const float* __restrict__ lo,
                                                     double sigma, double alpha, const double* __restrict__ x,
                                                     double beta, double* __restrict__ y) {
@@ -146,19 +245,15 @@ __global__ void __launch_bounds__(256) k_spmv_hilo(int64_t n, int k, const int32
     const int64_t cb = (r / kSlice) * (int64_t)(kSlice * k) + (r % kSlice);
     const double w0 = (double)ld_stream(hi + vb) + (double)ld_stream(lo + vb);
     double xi[Q], acc[Q];
+    load_x<Q>(x, r, xi);
 #pragma unroll
     for (int q = 0; q < Q; q++) {
-        xi[q] = x[r * Q + q];
         acc[q] = w0 * xi[q];
     }
-#pragma unroll 4
-    for (int s = 0; s < k; s++) {
-        const int64_t j = ld_stream(col + cb + (int64_t)s * kSlice);
+    add_slots<Q, 0>(k, col + cb, x, acc, [&](int s) {
         const int64_t e = vb + (int64_t)(s + 1) * kSlice;
-        const double w = (double)ld_stream(hi + e) + (double)ld_stream(lo + e);
-#pragma unroll
-        for (int q = 0; q < Q; q++) acc[q] = fma(w, x[j * Q + q], acc[q]);
-    }
+        return (double)ld_stream(hi + e) + (double)ld_stream(lo + e);
+    });
 #pragma unroll
     for (int q = 0; q < Q; q++) {
         double out = alpha * (sigma * xi[q] - acc[q]);
@@ -170,8 +265,8 @@ __global__ void __launch_bounds__(256) k_spmv_hilo(int64_t n, int k, const int32
 template <int Q>
 mvgd_status launch_hilo(const mvgd_ell* L, double sigma, double alpha, const void* x, double beta, void* y,
                         cudaStream_t s) {
-    unsigned blocks = (unsigned)((L->n + 255) / 256);
-    k_spmv_hilo<Q><<<blocks, 256, 0, s>>>(L->n, L->k, L->col, static_cast<const float*>(L->val), L->val_lo,
+    const unsigned blocks = (unsigned)((L->n + kHiloThreads - 1) / kHiloThreads);
+    k_spmv_hilo<Q><<<blocks, kHiloThreads, 0, s>>>(L->n, L->k, L->col, static_cast<const float*>(L->val), L->val_lo,
                                           sigma, alpha, static_cast<const double*>(x), beta,
                                           static_cast<double*>(y));
     return launch_status();
