@@ -65,7 +65,6 @@ class Pipeline:
             k += 1                                   # row scaling
         if self.precond == LB.PRECOND_AMG:
             k += amg_setup_kernels(self.n)
-            k += (lv - 2 if lv > 2 else 0) + 1       # level and coarsest chunk tables
         return k
 
     def run(self, pts: torch.Tensor, f: torch.Tensor) -> torch.Tensor:
