@@ -17,9 +17,9 @@ CSRC = PKG / "csrc"
 INCLUDE = ROOT / "include"
 OUT_DIR = PKG / "_build"
 LIB = OUT_DIR / "libmvgd.so"
-SOURCES = ("solve_mixed_amg.cu", "solve_fp64_amg.cu", "solve_mixed_plain.cu", "solve_fp64_plain.cu", "knn.cu",
-           "assemble.cu", "spmv.cu", "solve.cu", "amg.cu", "block.cu", "gs.cu", "neumann.cu", "capi.cu",
-           "ritz.cu")
+SOURCES = ("solve_mixed_amg.cu", "solve_fp64_amg.cu", "solve_mixed_amg_wide.cu", "solve_fp64_amg_wide.cu",
+           "solve_mixed_plain.cu", "solve_fp64_plain.cu", "knn.cu", "assemble.cu", "spmv.cu", "solve.cu", "amg.cu",
+           "block.cu", "gs.cu", "neumann.cu", "capi.cu", "ritz.cu")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
               "--expt-relaxed-constexpr"]

@@ -1767,6 +1767,11 @@ mvgd_status launch_solve(const ReqTable& tab, Ctl ctl, int budget, int kmax, cud
     return launch_solve_as<MIXED, QT, AMG, S_SINGLE>(tab, ctl, budget, kmax, s);
 }
 
+// The multigrid flows' widest instantiations, which take a third of their build, have
+// translation units of their own (solve_*_amg_wide.cu).
+extern template mvgd_status launch_solve<true, 8, true>(const ReqTable&, Ctl, int, int, cudaStream_t);
+extern template mvgd_status launch_solve<false, 8, true>(const ReqTable&, Ctl, int, int, cudaStream_t);
+
 template <bool MIXED, bool AMG>
 mvgd_status dispatch_q(int Q, const ReqTable& tab, Ctl ctl, int budget, int kmax, cudaStream_t s) {
     if (Q <= 1) return launch_solve<MIXED, 1, AMG>(tab, ctl, budget, kmax, s);
