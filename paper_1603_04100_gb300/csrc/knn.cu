@@ -129,14 +129,17 @@ __device__ __forceinline__ int cell_of(float x, float inv_s, int D) {
     return t > (float)(D - 1) ? D - 1 : (int)t;
 }
 
-// Cell coordinates as one word (at most 2^20 cells an axis).
+// Cell coordinates -1 .. 2^20 - 1 as one word, 21 bits each.  An axis whose extent is
+// not finite has no cells (D = 0) and its points the coordinate -1: such a query finds
+// no range and no ring to grow, and its list is empty (-1).  Packed as it is, -1 would
+// fill the word, and the ring sizes formed from it run into 10^8 rounds a query.
 __device__ __forceinline__ uint64_t pack_cell(const int (&c)[3]) {
-    return (uint64_t)c[0] | (uint64_t)c[1] << 21 | (uint64_t)c[2] << 42;
+    return (uint64_t)(c[0] + 1) | (uint64_t)(c[1] + 1) << 21 | (uint64_t)(c[2] + 1) << 42;
 }
 __device__ __forceinline__ void unpack_cell(uint64_t w, int (&c)[3]) {
-    c[0] = (int)(w & 0x1fffffu);
-    c[1] = (int)((w >> 21) & 0x1fffffu);
-    c[2] = (int)(w >> 42);
+    c[0] = (int)(w & 0x1fffffu) - 1;
+    c[1] = (int)((w >> 21) & 0x1fffffu) - 1;
+    c[2] = (int)(w >> 42) - 1;
 }
 
 // True in the last block of the grid to arrive (every thread of the block
@@ -283,7 +286,7 @@ __device__ void set_params(const unsigned* bits, int64_t n, int k, double cell_s
     for (int a = 0; a < 3; a++) {
         double d = floor(P->ext[a] * inv_s) + 1.0;
         if (d > 1048576.0) d = 1048576.0;
-        P->D[a] = (int)d;
+        P->D[a] = d >= 0.0 ? (int)d : 0;  // (no finite extent: an infinite coordinate, or none that is a number)
         int b = 0;
         while ((1 << b) < P->D[a] && b < 20) b++;
         Mb[a] = b < 2 ? 2 : b;  // wrap >= 4 so a 3-cell block never aliases

@@ -1,0 +1,63 @@
+"""kNN at the limits of its input: extents that are not finite."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_1603_04100_gb300 import inputs as I
+from tests.gpu_util import cuda_or_skip
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _spoilt(kind):
+    p = I.random_sphere(3000, 30)
+    axis = {"x": 0, "y": 1, "z": 2}[kind[0]]
+    if kind[1:] == "+inf":
+        p[17, axis] = np.inf
+    elif kind[1:] == "-inf":
+        p[17, axis] = -np.inf
+    elif kind[1:] == "inf both":
+        p[17, axis], p[2040, axis] = np.inf, -np.inf
+    elif kind[1:] == "overflow":  # finite points, an extent beyond FP64
+        p[17, axis], p[2040, axis] = 1.7e308, -1.7e308
+    else:
+        p[:, axis] = np.nan
+    return p
+
+
+@pytest.mark.parametrize("kind", [a + b for a in "xyz" for b in ("+inf", "-inf", "inf both", "overflow", "nan")])
+def test_extent_that_is_not_finite_gives_empty_lists(kind):
+    """No cell grid exists: the lists come back empty, the rows as not finite, and the
+    next cloud's lists are right."""
+    dev = cuda_or_skip()
+    from paper_1603_04100_gb300 import api
+    pt = torch.from_numpy(_spoilt(kind)).to(dev)
+    nbr, order = api.knn(pt, 20, want_order=True)
+    assert bool((nbr == -1).all())
+    assert torch.equal(torch.sort(order).values, torch.arange(len(pt), dtype=torch.int32, device=dev))
+    for prec in (api.FP64, api.FP32_REFINE):
+        op = api.assemble(pt, nbr, prec=prec, order=order)
+        assert int(op.bad_rows.item()) == len(pt) and bool((op.status == 2).all())
+    good = torch.from_numpy(I.random_sphere(3000, 30)).to(dev)
+    assert int(api.knn(good, 20).min()) >= 0
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_a_few_points_that_are_not_numbers_leave_the_others_exact(value):
+    """NaN coordinates are outside the box (an infinite one empties every list): the
+    other points' lists are those of the cloud without them."""
+    dev = cuda_or_skip()
+    from paper_1603_04100_gb300 import api
+    p = I.random_sphere(3000, 31)
+    bad = np.array([5, 1200, 2999])
+    q = p.copy()
+    q[bad] = value
+    nbr = api.knn(torch.from_numpy(q).to(dev), 12).cpu().numpy()
+    if np.isinf(value):
+        assert (nbr == -1).all()
+        return
+    keep = np.setdiff1d(np.arange(3000), bad)
+    want = api.knn(torch.from_numpy(np.ascontiguousarray(p[keep])).to(dev), 12).cpu().numpy()
+    np.testing.assert_array_equal(nbr[keep], keep[want])
