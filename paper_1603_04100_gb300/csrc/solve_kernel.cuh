@@ -1350,6 +1350,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
         masks(ph);
     };
     if constexpr (LOCAL) enter(0, P_PRE_A);
+    int stop_word = 0;  // LOCAL: the stop word at the end of the last iteration
 
     // One Krylov phase over every request's level-0 tiles, then the grid barrier.
     // the step that ends an iteration: it restarts the Krylov vectors of the
@@ -1465,6 +1466,8 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
                                   !(ctl.withhold && blockIdx.x == 0 && bar_epoch == 0));
         trace_step(ctl, (unsigned)ph);
         if constexpr (LOCAL) {
+            // (loaded with the partials: no round trip of its own)
+            if (ph == ph_end) stop_word = *(const volatile int*)ctl.stop;
             if (reduce && ok) local_advance(ph);
         }
         return ok;
@@ -1656,8 +1659,13 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     };
 
     // the counts are stable between the barrier that follows their last change and the
-    // next reducing step: identical in every block
-    auto finished = [&]() { return *(volatile int*)ctl.active == 0 || *(volatile int*)ctl.stop != 0; };
+    // next reducing step: identical in every block.  A launch that is told to stop leaves
+    // at an iteration's end, before the next PRE_A: what PRE_A applies (a pending step, a
+    // new p, the fold into u) the saved states still ask for, and a later launch of the
+    // same request would apply it again.  LOCAL reads its count behind PRE_A, but leaves
+    // there only with every right-hand side done, when PRE_A changes nothing.
+    auto finished = [&]() { return *(volatile int*)ctl.active == 0; };
+    auto stopped = [&]() { return LOCAL ? stop_word != 0 : *(volatile int*)ctl.stop != 0; };
     int running = -1;  // the launch's running right-hand sides when the list was formed
     for (int it = 0; it < iter_budget; ++it) {
         bool ok = true, leave = false;
@@ -1689,7 +1697,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
             }
         }
         if (!ok || leave) break;  // (an error exit: after the drain below)
-        if (!LOCAL && finished()) break;
+        if (stopped() || (!LOCAL && finished())) break;
     }
     if (LOCAL && bid == 0 && fit && tid < MVGD_NQ(sP)) sP.st[tid] = S[tid];
     // copies still landing (a missed wait): bounded waits before the block's
