@@ -347,14 +347,31 @@ __global__ void k_amg_dense(const AmgHeader* __restrict__ Hp, OpView O) {
         row2[c] = split_f2(v);
     };
     if (m == 0) {
-        if (lane != 0) return;  // a folded operator's columns may repeat: one after the other
+        // a lane a slot.  A folded operator's row may name a column twice, or itself (a
+        // point beside its ghost): such slots add up, in slot order, as in its products
+        static_assert(kMaxK + 1 <= kWarp, "a lane a slot");
         const int k = H.k;
         const int64_t vb = (r / kSlice) * (int64_t)(kSlice * (k + 1)) + (r % kSlice);
-        put(r, H.sigma - op_weight(O, vb));
-        for (int s = 0; s < k; s++) {
-            const int64_t j = O.col[(r / kSlice) * (int64_t)(kSlice * k) + (int64_t)s * kSlice + (r % kSlice)];
-            put(j, -op_weight(O, vb + (int64_t)(s + 1) * kSlice));
+        const int64_t cb = (r / kSlice) * (int64_t)(kSlice * k) + (r % kSlice);
+        int c = -1 - lane;  // (no slot)
+        double v = 0.0;
+        if (lane == 0) {
+            c = (int)r;
+            v = H.sigma - op_weight(O, vb);
+        } else if (lane <= k) {
+            c = O.col[cb + (int64_t)(lane - 1) * kSlice];
+            v = -op_weight(O, vb + (int64_t)lane * kSlice);
         }
+        unsigned rest = __match_any_sync(0xffffffffu, c);
+        const bool first = (rest & ((1u << lane) - 1u)) == 0;
+        double t = v;
+        rest &= rest - 1u;  // the slots that follow the column's first
+        while (__any_sync(0xffffffffu, rest != 0u)) {
+            const double x = __shfl_sync(0xffffffffu, v, rest ? __ffs(rest) - 1 : lane);
+            if (rest) t += x;
+            rest &= rest - 1u;
+        }
+        if (first && c >= 0) put(c, t);
     } else {
         const AmgLevel& L = H.lv[m];
         const int64_t b = (r / kSlice) * (int64_t)(kSlice * kAmgStride) + (r % kSlice);
