@@ -726,6 +726,12 @@ __device__ __forceinline__ double exact_d2(const double* __restrict__ pts, int i
     return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
+// FP32 squares and their sums round by at most half of 2^-149 where they are subnormal
+// (clouds of an extent near 1e-20), which no relative bound covers: an absolute error
+// bound of a squared distance, several times the three roundings.  Lost in the rounding
+// of any normal number above 2^-122.
+constexpr float kTinySq = 0x1p-146f;
+
 // Scan the block of ring R around cell c; returns the running list.
 template <bool EXACT>
 __device__ Key scan_block(const double* __restrict__ pts, const float4* __restrict__ sorted,
@@ -834,7 +840,7 @@ __device__ __noinline__ Key query_general(const double* __restrict__ pts, const 
         if (!exact_mode) {
             Key last = key_shfl(list, 31);
             if (last.b != 0xffffffffu) {
-                float d = __fsqrt_rd(__uint_as_float((uint32_t)last.a));
+                float d = __fsqrt_rd(fmaxf(__fsub_rd(__uint_as_float((uint32_t)last.a), kTinySq), 0.0f));
                 float lb = __fsub_rd(__fmul_rd(d, 1.0f - 8.0f * 5.9604645e-08f), p.eps_abs);
                 ex_ok = lb > ub;
             }
@@ -970,14 +976,15 @@ k_query(const double* __restrict__ pts, int64_t n, int k, const KnnParams* __res
                     list = warp_merge_words(list, warp_sort_words(key, lane), lane);
             }
             // the 32 smallest's FP32 squared distances with the bound on their error:
-            // |d_fp32 - d| <= eps from the coordinates, 4 roundings in the square
+            // |d_fp32 - d| <= eps from the coordinates, 4 roundings in the square (and, where
+            // they are subnormal, kTinySq)
             const bool have = list != 0xffffffffu;
             const float4 v = __ldg(&sorted[have ? qpos[list & kKeptMask] : (int)q]);
             const float dx = v.x - me.x, dyy = v.y - me.y, dzz = v.z - me.z;
             const float d2 = fmaf(dzz, dzz, fmaf(dyy, dyy, dx * dx));
             auto bound = [&](float x) {
-                const float d = sqrtf(x) * 1.000001f;
-                return (fmaf(2.0f, d, eps) * eps + x * (8.0f * 5.9604645e-08f)) * 1.001f;
+                const float d = sqrtf(x + kTinySq) * 1.000001f;
+                return (fmaf(2.0f, d, eps) * eps + x * (8.0f * 5.9604645e-08f)) * 1.001f + 2.0f * kTinySq;
             };
             const float err = bound(d2);
             const float lo = __fsub_rd(d2, err), hi = __fadd_ru(d2, err);
@@ -986,7 +993,7 @@ k_query(const double* __restrict__ pts, int64_t n, int k, const KnnParams* __res
             // guard, those screened out have keys above the last one kept
             const float out2 = __fmul_rd(fmaxf(__fsub_rd(__fmul_rd(guard, 1.0f - 8.0f * 5.9604645e-08f), eps), 0.0f),
                                          1.0f - 8.0f * 5.9604645e-08f);
-            float out_lo = open ? __fmul_rd(out2, out2) : FLT_MAX;
+            float out_lo = open ? __fsub_rd(__fmul_rd(out2, out2), 2.0f * kTinySq) : FLT_MAX;
             if (kept > 32) {
                 const float x = __uint_as_float(__shfl_sync(0xffffffffu, list, 31) & ~kKeptMask);
                 out_lo = fminf(out_lo, __fsub_rd(x, bound(x)));

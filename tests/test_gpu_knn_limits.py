@@ -1,9 +1,11 @@
-"""kNN at the limits of its input: extents that are not finite."""
+"""kNN at the limits of its input: extents that are not finite, clouds so small or large
+that FP32 squares of their distances are not normal numbers."""
 from __future__ import annotations
 
 import numpy as np
 import pytest
 
+import oracle
 from paper_1603_04100_gb300 import inputs as I
 from tests.gpu_util import cuda_or_skip
 
@@ -61,3 +63,15 @@ def test_a_few_points_that_are_not_numbers_leave_the_others_exact(value):
     keep = np.setdiff1d(np.arange(3000), bad)
     want = api.knn(torch.from_numpy(np.ascontiguousarray(p[keep])).to(dev), 12).cpu().numpy()
     np.testing.assert_array_equal(nbr[keep], keep[want])
+
+
+@pytest.mark.parametrize("k", [6, 20, 31])
+@pytest.mark.parametrize("scale", [1e-16, 1e-18, 1e-19, 3e-20, 1e-20, 3e-21, 1e-21, 1e-22, 1e-24, 1e-35, 1e15, 1e19, 1e25])
+def test_lists_are_exact_where_fp32_squares_underflow_or_overflow(scale, k):
+    """Squared distances that are subnormal (or zero, or infinite) in FP32: the screen's
+    bound has to know their absolute error."""
+    dev = cuda_or_skip()
+    from paper_1603_04100_gb300 import api
+    p = scale * I.random_sphere(2500, 32)
+    nbr = api.knn(torch.from_numpy(p).to(dev), k).cpu().numpy()
+    np.testing.assert_array_equal(nbr, oracle.knn_brute(p, k))
