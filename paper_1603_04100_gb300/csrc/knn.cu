@@ -20,7 +20,8 @@
 //      candidate's place in the warp's list, and the 32 smallest are sorted
 //      across lanes.  A compare-exchange is a shuffle and a min or max (96-bit
 //      (distance, index) keys took some fifteen instructions, for all of a
-//      block's candidates, and the integer pipe bound the kernel);
+//      block's candidates, and the integer pipe bound the kernel); past 256
+//      candidates the list is cut to the 32 smallest whenever it is full;
 //   3. proof: the kept candidates' FP32 distances with a bound on their error
 //      settle the order of the K nearest, and that no other point is nearer;
 //   4. where only the order is unsettled (distances closer than the bound), the
@@ -799,14 +800,15 @@ __device__ Key scan_block(const double* __restrict__ pts, const float4* __restri
 
 // The general query: rings double until the k-th distance is inside the block;
 // a block of more than M cells per axis visits each residue once, so every
-// scan is bounded by the bucket count and the loop by log2 of the grid size.
+// scan is bounded by the bucket count and the loop by log2 of the grid size.  The
+// first ring and whether FP32 keys are worth trying are what the screen has found.
 __device__ __noinline__ Key query_general(const double* __restrict__ pts, const float4* __restrict__ sorted,
                                           const int* __restrict__ start, const KnnParams& p, int k, int i, float4 me,
-                                          int c0, int c1, int c2) {
+                                          uint64_t cell, int ring, bool exact_mode) {
     const float qv[3] = {me.x, me.y, me.z};
-    const int c[3] = {c0, c1, c2};
-    bool exact_mode = false;
-    for (int R = 1;;) {
+    int c[3];
+    unpack_cell(cell, c);
+    for (int R = ring;;) {
         AxisRange ax[3];
         bool all_full = true;
         float guard = FLT_MAX;
@@ -879,10 +881,75 @@ __device__ __forceinline__ uint32_t warp_merge_words(uint32_t list, uint32_t chu
     return v;
 }
 
-constexpr int kKept = 256;  // candidates inside the guard a warp can hold; more: the general scan
+constexpr int kKept = 256;  // candidates inside the guard a warp can hold
 constexpr uint32_t kKeptMask = kKept - 1;
 
-__global__ void __launch_bounds__(kQueryWarps * 32)
+// The 32 smallest of a warp's `kept` keys, ascending.
+__device__ __forceinline__ uint32_t smallest_kept(const uint32_t* qkey, int kept, unsigned lane) {
+    uint32_t list = (int)lane < kept ? qkey[lane] : 0xffffffffu;
+    list = warp_sort_words(list, lane);
+    for (int t0 = 32; t0 < kept; t0 += 32) {
+        const uint32_t key = t0 + (int)lane < kept ? qkey[t0 + lane] : 0xffffffffu;
+        if (__any_sync(0xffffffffu, key < __shfl_sync(0xffffffffu, list, 31)))
+            list = warp_merge_words(list, warp_sort_words(key, lane), lane);
+    }
+    return list;
+}
+
+// The screen of a query with more candidates in its cells than a warp holds: points
+// denser than the cells were sized for (a graded or clustered cloud).  A full list is cut
+// down to its 32 smallest, and candidates at or above the last of those are dropped from
+// there on.  `off` and `shift`: the lanes' ranges; `cut`: the guard's square, as the
+// unsigned word whose order is that of non-negative floats.  Returns the candidates held.
+// A function of its own, so that ordinary queries keep their registers.  In ms a call,
+// 300,000 points most of which lie near two poles, K = 20 and 31: 2.6 and 5.2 (handed
+// to the general scan and its 96-bit keys: 5.1 and 8.2; by the general scan alone, before
+// there was a screen: 3.7 and 4.9).
+__device__ __noinline__ int screen_dense(const float4* __restrict__ sorted, float4 me, int off, int shift,
+                                         uint32_t cut, uint32_t* qkey, int* qpos) {
+    const unsigned lane = lane_id();
+    const int total = __shfl_sync(0xffffffffu, off, 31);
+    int kept = 0;
+    for (int t0 = 0; t0 < total; t0 += 32) {
+        const int t = t0 + (int)lane;
+        int l = 0;
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1)
+            if (__shfl_sync(0xffffffffu, off, l + step - 1) <= t) l += step;
+        const int pos = t + __shfl_sync(0xffffffffu, shift, l & 31);
+        uint32_t d2 = 0xffffffffu;
+        if (t < total) {
+            const float4 v = __ldg(&sorted[pos]);
+            const float dx = v.x - me.x, dy = v.y - me.y, dz = v.z - me.z;
+            if (__float_as_int(v.w) != __float_as_int(me.w))
+                d2 = __float_as_uint(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
+        }
+        unsigned who = __ballot_sync(0xffffffffu, d2 < cut);
+        if (kept + __popc(who) > kKept) {
+            __syncwarp();
+            const uint32_t list = smallest_kept(qkey, kept, lane);
+            const int at = qpos[list & kKeptMask];
+            __syncwarp();
+            qkey[lane] = (list & ~kKeptMask) | lane;
+            qpos[lane] = at;
+            __syncwarp();
+            cut = min(cut, __shfl_sync(0xffffffffu, list, 31) & ~kKeptMask);
+            kept = 32;
+            who = __ballot_sync(0xffffffffu, d2 < cut);
+        }
+        if (d2 < cut) {
+            const int at = kept + __popc(who & ((1u << lane) - 1u));
+            qkey[at] = (d2 & ~kKeptMask) | (uint32_t)at;
+            qpos[at] = pos;
+        }
+        kept += __popc(who);
+    }
+    return kept;
+}
+
+// (four blocks an SM: with the 80 registers that three leave the call took 1.52 ms instead
+// of 1.31 at 1,048,576 points)
+__global__ void __launch_bounds__(kQueryWarps * 32, 4)
 k_query(const double* __restrict__ pts, int64_t n, int k, const KnnParams* __restrict__ P,
         const float4* __restrict__ sorted, const int* __restrict__ start, const uint64_t* __restrict__ scell,
         int32_t* __restrict__ nbr, int per_warp) {
@@ -924,7 +991,8 @@ k_query(const double* __restrict__ pts, int64_t n, int k, const KnnParams* __res
             const int v = __shfl_up_sync(0xffffffffu, off, o);
             if ((int)lane >= o) off += v;
         }
-        const int total = __shfl_sync(0xffffffffu, off, 31);
+        int total = __shfl_sync(0xffffffffu, off, 31);
+        total = total > kKept ? 0 : total;  // (more: screen_dense)
         const int shift = beg - (off - cnt);  // a candidate of this lane's range: its place + shift
         // the guard: the query's distance to the faces of the block, rounded down.  A K-th
         // neighbour beyond it needs more rings anyway, so candidates beyond it are dropped
@@ -957,24 +1025,24 @@ k_query(const double* __restrict__ pts, int64_t n, int k, const KnnParams* __res
                 keep = __float_as_int(v.w) != i && !(d2 >= guard2);
             }
             const unsigned who = __ballot_sync(0xffffffffu, keep);
-            const int at = kept + __popc(who & ((1u << lane) - 1u));
-            if (keep && at < kKept) {
+            if (keep) {
+                const int at = kept + __popc(who & ((1u << lane) - 1u));
                 qkey[at] = (__float_as_uint(d2) & ~kKeptMask) | (uint32_t)at;
                 qpos[at] = pos;
             }
             kept += __popc(who);
         }
+        if (__shfl_sync(0xffffffffu, off, 31) > kKept)
+            kept = screen_dense(sorted, me, off, shift, __float_as_uint(guard2), qkey, qpos);
         __syncwarp();
         int32_t nb = 0;
         bool done = false;
-        if (kept >= k && kept <= kKept) {
-            uint32_t list = (int)lane < kept ? qkey[lane] : 0xffffffffu;
-            list = warp_sort_words(list, lane);
-            for (int t0 = 32; t0 < kept; t0 += 32) {
-                const uint32_t key = t0 + (int)lane < kept ? qkey[t0 + lane] : 0xffffffffu;
-                if (__any_sync(0xffffffffu, key < __shfl_sync(0xffffffffu, list, 31)))
-                    list = warp_merge_words(list, warp_sort_words(key, lane), lane);
-            }
+        // the general scan's first ring (fewer than K inside the guard: the next one), and
+        // whether FP32 distances have already failed to tell the 32nd candidate from the K-th
+        int ring = open && kept < k ? 2 : 1;
+        bool tight = false;
+        if (kept >= k) {
+            const uint32_t list = smallest_kept(qkey, kept, lane);
             // the 32 smallest's FP32 squared distances with the bound on their error:
             // |d_fp32 - d| <= eps from the coordinates, 4 roundings in the square (and, where
             // they are subnormal, kTinySq)
@@ -994,9 +1062,11 @@ k_query(const double* __restrict__ pts, int64_t n, int k, const KnnParams* __res
             const float out2 = __fmul_rd(fmaxf(__fsub_rd(__fmul_rd(guard, 1.0f - 8.0f * 5.9604645e-08f), eps), 0.0f),
                                          1.0f - 8.0f * 5.9604645e-08f);
             float out_lo = open ? __fsub_rd(__fmul_rd(out2, out2), 2.0f * kTinySq) : FLT_MAX;
-            if (kept > 32) {
+            if (kept >= 32) {  // (32: a dense query's list may have been cut)
                 const float x = __uint_as_float(__shfl_sync(0xffffffffu, list, 31) & ~kKeptMask);
-                out_lo = fminf(out_lo, __fsub_rd(x, bound(x)));
+                const float x_lo = __fsub_rd(x, bound(x));
+                out_lo = fminf(out_lo, x_lo);
+                tight = !(x_lo > kth_hi);
             }
             const float prev = __shfl_up_sync(0xffffffffu, hi, 1);
             const bool settled = lane == 0 || !have || ((int)lane < k ? lo > prev : lo > kth_hi);
@@ -1018,7 +1088,7 @@ k_query(const double* __restrict__ pts, int64_t n, int k, const KnnParams* __res
                 }
             }
         }
-        if (!done) nb = (int32_t)query_general(pts, sorted, start, p, k, i, me, c[0], c[1], c[2]).b;
+        if (!done) nb = (int32_t)query_general(pts, sorted, start, p, k, i, me, scell[q], ring, tight).b;
         if ((int)lane < k) nbr[(int64_t)i * k + lane] = nb;
         __syncwarp();  // the kept lists are read; the next query may write them
     }

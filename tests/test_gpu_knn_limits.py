@@ -1,5 +1,6 @@
 """kNN at the limits of its input: extents that are not finite, clouds so small or large
-that FP32 squares of their distances are not normal numbers."""
+that FP32 squares of their distances are not normal numbers, and points far denser
+than the search grid."""
 from __future__ import annotations
 
 import numpy as np
@@ -75,3 +76,26 @@ def test_lists_are_exact_where_fp32_squares_underflow_or_overflow(scale, k):
     p = scale * I.random_sphere(2500, 32)
     nbr = api.knn(torch.from_numpy(p).to(dev), k).cpu().numpy()
     np.testing.assert_array_equal(nbr, oracle.knn_brute(p, k))
+
+
+def _graded(n, seed):  # a sphere whose points crowd at two poles
+    p = I.random_sphere(n, seed)
+    z = np.sign(p[:, 2]) * (1 - (1 - np.abs(p[:, 2])) ** 3)
+    rho = np.sqrt(np.maximum(1 - z * z, 0)) / np.hypot(p[:, 0], p[:, 1])
+    return np.ascontiguousarray(np.stack([p[:, 0] * rho, p[:, 1] * rho, z], 1))
+
+
+@pytest.mark.parametrize("k", [1, 20, 31])
+@pytest.mark.parametrize("cell", [0.0, -2.0, 0.06, 0.4])
+def test_queries_with_more_candidates_than_a_warp_holds(cell, k):
+    """From a few hundred candidates in a query's cells to thousands inside its guard,
+    ties and points that are not numbers among them."""
+    dev = cuda_or_skip()
+    from paper_1603_04100_gb300 import api
+    p = _graded(6000, 33)
+    p[100:140] = p[99]
+    nbr = api.knn(torch.from_numpy(p).to(dev), k, cell_size=cell).cpu().numpy()
+    np.testing.assert_array_equal(nbr, oracle.knn_brute(p, k))
+    q = np.concatenate([p, np.full((50, 3), np.nan)])
+    nbr = api.knn(torch.from_numpy(q).to(dev), k, cell_size=cell).cpu().numpy()
+    np.testing.assert_array_equal(nbr[:6000], oracle.knn_brute(p, k))
