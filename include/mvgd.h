@@ -503,6 +503,8 @@ mvgd_status mvgd_amg_apply(const void *amg_ws, int64_t n, int32_t nrhs, const do
  *   mvgd_iterate_workspace_bytes for at least this many requests and rows)
  *   holds the launch's tables and barrier.  Asynchronous; a set cancel word
  *   stops the launch after the current iteration.
+ *   A descriptor whose nrhs or k is not its request's ends the launch with
+ *   MVGD_EINVAL as the status of the right-hand sides not yet done.
  * mvgd_request_finish: writes u (FP64 [n][nrhs], point order) and info
  *   (DEVICE [nrhs]); a right-hand side not yet done reports MVGD_ENOCONV,
  *   or MVGD_ECANCELLED / MVGD_ETIMEOUT if a launch was cut short.
@@ -515,7 +517,7 @@ size_t mvgd_iterate_workspace_bytes(int32_t max_requests, int64_t max_total_rows
 typedef struct {
     void *workspace;  /* the request's workspace, as given to mvgd_request_init */
     int64_t n;        /* rows of its operator */
-    int32_t nrhs;     /* its right-hand sides */
+    int32_t nrhs;     /* its right-hand sides, as given to mvgd_request_init */
     int32_t k;        /* K of its operator (sizes the launch's shared-memory staging) */
 } mvgd_request;
 mvgd_status mvgd_iterate(const mvgd_request *reqs, int32_t count, int32_t prec, int32_t precond,

@@ -1206,9 +1206,12 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
         __syncthreads();
         const Prob& P = sP;
         // a K above the one the staging buffers were sized for (a wrong K in the
-        // request list) would overrun shared memory, and a hierarchy of another
-        // operator would be read out of bounds: do no work and end the launch
-        bool fits = P.k <= kmax && ((P.amg != nullptr) == AMG);
+        // request list) would overrun shared memory, right-hand sides other than the
+        // list's would put a group's columns past the arrays or overrun the states,
+        // and a hierarchy of another operator would be read out of bounds: do no work
+        // and end the launch
+        bool fits = P.k <= kmax && ((P.amg != nullptr) == AMG) &&
+                    (tab.groups > 1 ? P.Q == tab.groups * tab.gq : P.Q <= tab.gq);
         if (AMG && fits) fits = P.amg->n == P.n && P.amg->k == P.k;
         if (!fits && tid == 0) atomicCAS(ctl.err, 0, (int)MVGD_EINVAL);
         fit = fits;
