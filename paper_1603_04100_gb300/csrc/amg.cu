@@ -904,8 +904,12 @@ MVGD_API mvgd_status mvgd_amg_setup(const mvgd_ell* L, double sigma, void* amg_w
     {
         const int ncta = (int)((nc + kInvCols - 1) / kInvCols);
         const size_t smem = sizeof(float) * inv_smem_floats((int)nc);
-        auto fn = nc <= kInvStepThreads ? k_amg_invert<1> : (nc <= 2 * kInvStepThreads ? k_amg_invert<2> : k_amg_invert<4>);
-        MVGD_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const int rows = nc <= kInvStepThreads ? 1 : (nc <= 2 * kInvStepThreads ? 2 : 4);
+        auto fn = rows == 1 ? k_amg_invert<1> : (rows == 2 ? k_amg_invert<2> : k_amg_invert<4>);
+        // the instantiation's largest, whatever this level needs: the attribute is the
+        // process's, and another thread may be setting up a smaller level
+        const int most = (int)(sizeof(float) * inv_smem_floats(rows * kInvStepThreads));
+        MVGD_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)ncta);
         cfg.blockDim = dim3(kInvThreads);

@@ -44,6 +44,7 @@
 // refinement does not settle, or with a non-finite value or an invalid
 // neighbour index is handed to the FP64 path (k_assemble_fix), which also
 // sets its row_status.
+#include <algorithm>
 #include <type_traits>
 #include <vector>
 
@@ -777,6 +778,14 @@ bool fp32_path(const mvgd_ell& L, const mvgd_delta_rule& rule) {
     return L.prec == MVGD_FP32_REFINE && rule.arith == 0 && L.k >= kMinKMixed;
 }
 
+// What the kernels' launches may ask for: their largest, whatever the call needs (the
+// attribute is the process's, and another thread may be assembling with a smaller K).
+constexpr size_t kMixedMax = 200 << 10;  // of a block's warps together
+template <typename F>
+bool allow_smem(F* kernel, size_t bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+}
+
 constexpr int kFixBlocks = 152;  // grid of the hand-over kernels (a warp each)
 
 }  // namespace
@@ -830,19 +839,19 @@ MVGD_API mvgd_status mvgd_assemble(const double* pts, int64_t n, int32_t k, cons
     // resident warps)
     int wpb = mixed ? tuned_assemble_warps() : 1;
     const size_t per_warp = mixed ? smem_mixed(k) : smem_fp64(k);
-    while (wpb > 1 && per_warp * wpb > (size_t)(200 << 10)) wpb >>= 1;
+    while (wpb > 1 && per_warp * wpb > kMixedMax) wpb >>= 1;
     const unsigned blocks = (unsigned)((nslices + wpb - 1) / wpb);
     if (mixed) {
         MVGD_CUDA_TRY(cudaMemsetAsync(W.nfix, 0, sizeof(int32_t), s));
         const size_t sm = per_warp * wpb;
-        MVGD_CUDA_TRY(cudaFuncSetAttribute(k_assemble<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        if (!allow_smem(k_assemble<1>, kMixedMax)) return MVGD_ECUDA;
         k_assemble<1><<<blocks, kWarp * wpb, sm, s>>>(A);
         const size_t sf = smem_fp64(k);
-        MVGD_CUDA_TRY(cudaFuncSetAttribute(k_assemble_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sf));
+        if (!allow_smem(k_assemble_fix, smem_fp64(kMaxK))) return MVGD_ECUDA;
         k_assemble_fix<<<kFixBlocks, kWarp, sf, s>>>(A);
     } else {
         const size_t sf = per_warp * wpb;
-        MVGD_CUDA_TRY(cudaFuncSetAttribute(k_assemble<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sf));
+        if (!allow_smem(k_assemble<0>, smem_fp64(kMaxK))) return MVGD_ECUDA;
         k_assemble<0><<<blocks, kWarp * wpb, sf, s>>>(A);
     }
     return launch_status();
@@ -948,10 +957,10 @@ MVGD_API mvgd_status mvgd_assemble_batch(const mvgd_assemble_item* items, int32_
     if (slices >= (1ll << 31)) return MVGD_EINVAL;
     const size_t sf = smem_fp64(kmax), sm = smem_mixed(kmax);
     const size_t smem = any_fp64 ? (sf > sm ? sf : sm) : sm;
-    MVGD_CUDA_TRY(cudaFuncSetAttribute(k_assemble_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (!allow_smem(k_assemble_batch, std::max(smem_fp64(kMaxK), smem_mixed(kMaxK)))) return MVGD_ECUDA;
     k_assemble_batch<<<(unsigned)slices, kWarp, smem, s>>>(table, count);
     if (any_mixed) {
-        MVGD_CUDA_TRY(cudaFuncSetAttribute(k_assemble_batch_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sf));
+        if (!allow_smem(k_assemble_batch_fix, smem_fp64(kMaxK))) return MVGD_ECUDA;
         k_assemble_batch_fix<<<kFixBlocks, kWarp, sf, s>>>(table, fix, nfix);
     }
     return launch_status();

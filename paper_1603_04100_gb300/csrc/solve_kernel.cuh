@@ -1708,6 +1708,14 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     st.drain(MVGD_STAGE_BAR);
 }
 
+// The dynamic shared memory that an instantiation's launches may ask for, set to the
+// largest any of them does and not to the launch's own: a kernel's attribute is the
+// process's, and another thread's smaller launch could lower it between this one's set
+// and its launch.
+constexpr size_t kStageMax = 112 << 10;  // two buffers a warp, at most
+constexpr size_t kDynamicMax = kStageMax + kActBytes;
+static_assert(stage_bytes_per_warp<double>(kMaxK) * (kThreads / kWarp) <= kStageMax, "one buffer a warp always fits");
+
 // Slice buffers per warp.  One by default: a second buffer (the next tile's
 // slice requested ahead) costs a resident block per SM, and on GB300 at 1M
 // rows, K = 20, three single-buffered blocks ran the FP32 multigrid solve 8 %
@@ -1715,7 +1723,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
 // loses the third block's latency hiding).  mvgd_set_launch_tuning selects two.
 template <typename VT>
 int stage_buffers(int kmax) {
-    if (tuned_stage_buffers() == 2 && 2 * stage_bytes_per_warp<VT>(kmax) * (kThreads / kWarp) <= (112u << 10))
+    if (tuned_stage_buffers() == 2 && 2 * stage_bytes_per_warp<VT>(kmax) * (kThreads / kWarp) <= kStageMax)
         return 2;
     return 1;
 }
@@ -1729,7 +1737,7 @@ int solve_capacity(int kmax, size_t* smem_out = nullptr, size_t more = 0) {
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynamicMax) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem) != cudaSuccess)
         return 0;
     const int want = tuned_solver_blocks_per_sm();
