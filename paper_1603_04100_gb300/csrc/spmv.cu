@@ -9,6 +9,8 @@
 //             rows of L sum to zero, so the self weight is implied and the
 //             products act on small differences of a smooth vector;
 //   F64_HILO  standard form with w = hi + lo evaluated in FP64.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace mvgd {
@@ -82,70 +84,73 @@ __device__ __forceinline__ void load_x(const float* __restrict__ x, int64_t j, f
 // Rows a block of the FP64 products.  With several right-hand sides they are bound by the
 // FP64 pipe (2 FMAs a clock an SM), and blocks of 256 leave some SMs a third more rows than
 // others (100,003 rows: 391 blocks on 152 SMs); one warp a block spreads them within 3 %
-// and a small operator over every SM.  A block of a warp also caps an SM at 32 warps, which
-// costs nothing where K is fixed at compile time and a row's loads are issued ahead, but does
-// with the loop over a K known at run time (524,288 rows, K = 30, one vector: 40 us with 256
-// threads, 45 with 32), which keeps 256.  The hi + lo product has two FP64 conversions and an
-// addition a weight more on that pipe and gains at every K (1,048,576 rows, K = 20:
-// 177 -> 172 us; 524,288, K = 31: 141 -> 131).
-constexpr int spmv_threads(int kk) { return kk > 0 ? 32 : 256; }
-constexpr int kHiloThreads = 32;
+// and a small operator over every SM.  The hi + lo product has two FP64 conversions and an
+// addition a weight more on that pipe and gains with a loop over K too (1,048,576 rows,
+// K = 20: 177 -> 172 us; 524,288, K = 31: 141 -> 131).
+constexpr int kF64Threads = 32;
 
-// acc += the row's k slots in order, `weight(s)` times row col[s * kSlice] of x.  K fixed at
-// compile time: the columns, weights and rows of x of a batch are all requested before the
-// first product.  Else the compiler's unrolling, with wide loads of x only for eight vectors
-// (100,003 rows, K = 30, four: 32.7 us without, 33.4 with; 524,288 rows, eight: 277, 246).
-// In us, before (scalar loads, blocks of 256) -> now: 20,001 rows, K = 20, eight vectors
-// 25 -> 16; 524,288 rows, K = 24, eight 230 -> 197; 100,003 rows, K = 16, four 20.5 -> 20.0
-// (12 of them the FP64 pipe); 20,001 rows, K = 31, one 16 -> 6.2.
-template <int Q, int KK, typename Weight>
-__device__ __forceinline__ void add_slots(int k, const int32_t* __restrict__ col, const double* __restrict__ x,
-                                          double (&acc)[Q], Weight&& weight) {
-    constexpr int B = Q <= 2 ? 8 : 4;
-    int s0 = 0;
-    if constexpr (KK > 0) {
-#pragma unroll (KK / B)
-        for (; s0 + B <= KK; s0 += B) {
-            int32_t c[B];
-            double w[B], xj[B][Q];
+// The row's k slots in order, `add(weight, row of x)` for each: GROUPS = k / 4 groups of
+// four, known at compile time, and (REST) the k % 4 slots left over.  The columns, weights
+// and rows of x of a batch of BATCH slots are all requested before its first product,
+// whatever K is; a loop over a K known at run time keeps four slots' loads in flight.
+template <int Q, int GROUPS, bool REST, int BATCH, typename T, typename Add>
+__device__ __forceinline__ void walk_slots(int k, const int32_t* __restrict__ col, const T* __restrict__ val,
+                                           const T* __restrict__ x, Add&& add) {
+    auto batch = [&](auto width, int s0) {  // slots s0 .. s0 + width - 1
+        constexpr int W = decltype(width)::value;
+        int32_t c[W];
+        T w[W], xj[W][Q];
 #pragma unroll
-            for (int u = 0; u < B; u++) c[u] = ld_stream(col + (int64_t)(s0 + u) * kSlice);
+        for (int u = 0; u < W; u++) c[u] = ld_stream(col + (int64_t)(s0 + u) * kSlice);
 #pragma unroll
-            for (int u = 0; u < B; u++) w[u] = weight(s0 + u);
+        for (int u = 0; u < W; u++) w[u] = ld_stream(val + (int64_t)(s0 + u + 1) * kSlice);
 #pragma unroll
-            for (int u = 0; u < B; u++) load_x<Q>(x, c[u], xj[u]);
+        for (int u = 0; u < W; u++) load_x<Q>(x, c[u], xj[u]);
 #pragma unroll
-            for (int u = 0; u < B; u++)
+        for (int u = 0; u < W; u++) add(w[u], xj[u]);
+    };
+    constexpr int F = 4 * GROUPS;
 #pragma unroll
-                for (int q = 0; q < Q; q++) acc[q] = fma(w[u], xj[u][q], acc[q]);
-        }
-    }
-#pragma unroll 4
-    for (; s0 < k; s0++) {
-        const int64_t j = ld_stream(col + (int64_t)s0 * kSlice);
-        const double w = weight(s0);
-        double xj[Q];
-        if constexpr (KK > 0 || Q == 8) {
-            load_x<Q>(x, j, xj);
-        } else {
-#pragma unroll
-            for (int q = 0; q < Q; q++) xj[q] = x[j * Q + q];
-        }
-#pragma unroll
-        for (int q = 0; q < Q; q++) acc[q] = fma(w, xj[q], acc[q]);
+    for (int b = 0; b < F / BATCH; b++) batch(std::integral_constant<int, BATCH>{}, b * BATCH);
+    if constexpr (F % BATCH != 0) batch(std::integral_constant<int, F % BATCH>{}, F / BATCH * BATCH);
+    if constexpr (REST) {  // branches, not predicates: an FMA that is off still takes its turn on the pipe
+        const int rest = k - F;
+        if (rest == 1) batch(std::integral_constant<int, 1>{}, F);
+        else if (rest == 2) batch(std::integral_constant<int, 2>{}, F);
+        else if (rest == 3) batch(std::integral_constant<int, 3>{}, F);
     }
 }
 
-// KK > 0: K fixed at compile time (every slot's loads can be issued at once);
-// KK == 0: K at run time.
-template <int Q, int KK>
-__global__ void __launch_bounds__(spmv_threads(KK)) k_spmv_f64(int64_t n, int kr, const int32_t* __restrict__ col,
+// `launch(groups)` with groups = k / 4 at compile time.
+template <typename Launch>
+void by_groups(int k, Launch&& launch) {
+    static_assert(kMaxK / 4 == 7, "a case a group count");
+    switch (k / 4) {
+        case 0: launch(std::integral_constant<int, 0>{}); break;
+        case 1: launch(std::integral_constant<int, 1>{}); break;
+        case 2: launch(std::integral_constant<int, 2>{}); break;
+        case 3: launch(std::integral_constant<int, 3>{}); break;
+        case 4: launch(std::integral_constant<int, 4>{}); break;
+        case 5: launch(std::integral_constant<int, 5>{}); break;
+        case 6: launch(std::integral_constant<int, 6>{}); break;
+        default: launch(std::integral_constant<int, 7>{}); break;
+    }
+}
+
+// FP64, in us, against a loop over K of blocks of 256 rows with scalar loads of x: 20,001
+// rows, K = 18, one vector 5.0 -> 3.1, K = 31 7.9 -> 3.5, K = 20, eight 25 -> 16; 524,288
+// rows, K = 25, four vectors 108 -> 103, K = 24, eight 230 -> 197; 100,003 rows, K = 16,
+// four 20.5 -> 19.2 (12 of them the FP64 pipe), but K = 28, seven 47 -> 52 (its registers
+// leave a partial second wave there).
+// REST: K is not 4 GROUPS (else it is known at compile time: 5 % at 100,003 rows, K = 16).
+template <int Q, int GROUPS, bool REST>
+__global__ void __launch_bounds__(kF64Threads) k_spmv_f64(int64_t n, int kr, const int32_t* __restrict__ col,
                                                    const double* __restrict__ val, double sigma, double alpha,
                                                    const double* __restrict__ x, double beta,
                                                    double* __restrict__ y) {
     const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (r >= n) return;
-    const int k = KK > 0 ? KK : kr;
+    const int k = REST ? kr : 4 * GROUPS;
     const int m = k + 1;
     const int64_t vb = (r / kSlice) * (int64_t)(kSlice * m) + (r % kSlice);
     const int64_t cb = (r / kSlice) * (int64_t)(kSlice * k) + (r % kSlice);
@@ -156,7 +161,10 @@ __global__ void __launch_bounds__(spmv_threads(KK)) k_spmv_f64(int64_t n, int kr
     for (int q = 0; q < Q; q++) {
         acc[q] = w0 * xi[q];
     }
-    add_slots<Q, KK>(k, col + cb, x, acc, [&](int s) { return ld_stream(val + vb + (int64_t)(s + 1) * kSlice); });
+    walk_slots<Q, GROUPS, REST, (Q <= 2 ? 8 : 4)>(k, col + cb, val + vb, x, [&](double w, const double (&xj)[Q]) {
+#pragma unroll
+        for (int q = 0; q < Q; q++) acc[q] = fma(w, xj[q], acc[q]);
+    });
 #pragma unroll
     for (int q = 0; q < Q; q++) {
         double out = alpha * (sigma * xi[q] - acc[q]);
@@ -165,6 +173,10 @@ __global__ void __launch_bounds__(spmv_threads(KK)) k_spmv_f64(int64_t n, int kr
     }
 }
 
+// KK > 0: K fixed at compile time (the K of the workloads; every slot's loads can be issued
+// at once).  KK < 0: -KK - 1 groups of four and the rest, with up to three vectors: 20,001
+// rows, K = 25, one vector 5.2 -> 2.8 us, two 4.2 -> 3.2; 524,288 rows, K = 28, one 27 -> 20.
+// KK == 0: a loop over K, with more (K = 28, four, 100,003 rows: 9 us, 14 by groups).
 template <int Q, int KK>
 __global__ void __launch_bounds__(256) k_spmv_f32(int64_t n, int kr, const int32_t* __restrict__ col,
                                                    const float* __restrict__ val, float sigma, float alpha,
@@ -182,20 +194,20 @@ __global__ void __launch_bounds__(256) k_spmv_f32(int64_t n, int kr, const int32
     for (int q = 0; q < Q; q++) {
         acc[q] = 0.0f;
     }
-#pragma unroll (KK > 0 ? KK : 4)
-    for (int s = 0; s < k; s++) {
-        const int64_t j = ld_stream(col + cb + (int64_t)s * kSlice);
-        const float w = ld_stream(val + vb + (int64_t)(s + 1) * kSlice);
-        if constexpr (KK == 0 && (Q == 2 || Q == 3)) {
-            // (the row gathered into an array first, wide or not, the compiler keeps fewer
-            // slots' loads in flight: 20,001 rows, K = 28, two vectors 4.2 -> 7.3 us)
+    auto add = [&](float w, const float (&xj)[Q]) {
 #pragma unroll
-            for (int q = 0; q < Q; q++) acc[q] = fmaf(w, x[j * Q + q] - xi[q], acc[q]);
-        } else {
+        for (int q = 0; q < Q; q++) acc[q] = fmaf(w, xj[q] - xi[q], acc[q]);
+    };
+    if constexpr (KK < 0) {
+        walk_slots<Q, -KK - 1, true, 8>(k, col + cb, val + vb, x, add);
+    } else {
+#pragma unroll (KK > 0 ? KK : 4)
+        for (int s = 0; s < k; s++) {
+            const int64_t j = ld_stream(col + cb + (int64_t)s * kSlice);
+            const float w = ld_stream(val + vb + (int64_t)(s + 1) * kSlice);
             float xj[Q];
             load_x<Q>(x, j, xj);
-#pragma unroll
-            for (int q = 0; q < Q; q++) acc[q] = fmaf(w, xj[q] - xi[q], acc[q]);
+            add(w, xj);
         }
     }
 #pragma unroll
@@ -207,32 +219,37 @@ __global__ void __launch_bounds__(256) k_spmv_f32(int64_t n, int kr, const int32
 }
 
 template <int Q, int KK>
-void launch_spmv_k(const mvgd_ell* L, int mode, double sigma, double alpha, const void* x, double beta, void* y,
-                   cudaStream_t s) {
-    const int64_t n = L->n;
-    const unsigned blocks = (unsigned)((n + 255) / 256);
-    if (mode == MVGD_SPMV_F32)
-        k_spmv_f32<Q, KK><<<blocks, 256, 0, s>>>(n, L->k, L->col, static_cast<const float*>(L->val), (float)sigma,
-                                                 (float)alpha, static_cast<const float*>(x), (float)beta,
-                                                 static_cast<float*>(y));
-    else
-        k_spmv_f64<Q, KK><<<(unsigned)((n + spmv_threads(KK) - 1) / spmv_threads(KK)), spmv_threads(KK), 0, s>>>(n, L->k, L->col, static_cast<const double*>(L->val), sigma, alpha,
-                                                 static_cast<const double*>(x), beta, static_cast<double*>(y));
+void launch_f32(const mvgd_ell* L, double sigma, double alpha, const void* x, double beta, void* y, cudaStream_t s) {
+    k_spmv_f32<Q, KK><<<(unsigned)((L->n + 255) / 256), 256, 0, s>>>(
+        L->n, L->k, L->col, static_cast<const float*>(L->val), (float)sigma, (float)alpha,
+        static_cast<const float*>(x), (float)beta, static_cast<float*>(y));
+}
+
+template <int Q, int GROUPS>
+void launch_f64(const mvgd_ell* L, double sigma, double alpha, const void* x, double beta, void* y, cudaStream_t s) {
+    auto fn = L->k == 4 * GROUPS ? k_spmv_f64<Q, GROUPS, false> : k_spmv_f64<Q, GROUPS, true>;
+    fn<<<(unsigned)((L->n + kF64Threads - 1) / kF64Threads), kF64Threads, 0, s>>>(
+        L->n, L->k, L->col, static_cast<const double*>(L->val), sigma, alpha, static_cast<const double*>(x), beta,
+        static_cast<double*>(y));
 }
 
 template <int Q>
 mvgd_status launch_spmv(const mvgd_ell* L, int mode, double sigma, double alpha, const void* x, double beta,
                         void* y, cudaStream_t s) {
-    if (mode == MVGD_SPMV_F32 || mode == MVGD_SPMV_F64) {
-        // the common K and the largest at compile time, any other at run time
+    if (mode == MVGD_SPMV_F32) {
         switch (L->k) {
-            case 12: launch_spmv_k<Q, 12>(L, mode, sigma, alpha, x, beta, y, s); break;
-            case 16: launch_spmv_k<Q, 16>(L, mode, sigma, alpha, x, beta, y, s); break;
-            case 20: launch_spmv_k<Q, 20>(L, mode, sigma, alpha, x, beta, y, s); break;
-            case 24: launch_spmv_k<Q, 24>(L, mode, sigma, alpha, x, beta, y, s); break;
-            case 31: launch_spmv_k<Q, 31>(L, mode, sigma, alpha, x, beta, y, s); break;
-            default: launch_spmv_k<Q, 0>(L, mode, sigma, alpha, x, beta, y, s); break;
+            case 12: launch_f32<Q, 12>(L, sigma, alpha, x, beta, y, s); break;
+            case 16: launch_f32<Q, 16>(L, sigma, alpha, x, beta, y, s); break;
+            case 20: launch_f32<Q, 20>(L, sigma, alpha, x, beta, y, s); break;
+            case 24: launch_f32<Q, 24>(L, sigma, alpha, x, beta, y, s); break;
+            default:
+                if constexpr (Q <= 3)
+                    by_groups(L->k, [&](auto g) { launch_f32<Q, -decltype(g)::value - 1>(L, sigma, alpha, x, beta, y, s); });
+                else
+                    launch_f32<Q, 0>(L, sigma, alpha, x, beta, y, s);
         }
+    } else if (mode == MVGD_SPMV_F64) {
+        by_groups(L->k, [&](auto g) { launch_f64<Q, decltype(g)::value>(L, sigma, alpha, x, beta, y, s); });
     } else {
         // hi + lo: hi is stored as float in val; read it through a float view
         return MVGD_EINVAL;
@@ -241,7 +258,7 @@ mvgd_status launch_spmv(const mvgd_ell* L, int mode, double sigma, double alpha,
 }
 
 template <int Q>
-__global__ void __launch_bounds__(kHiloThreads) k_spmv_hilo(int64_t n, int k, const int32_t* __restrict__ col,
+__global__ void __launch_bounds__(kF64Threads) k_spmv_hilo(int64_t n, int k, const int32_t* __restrict__ col,
                                                     const float* __restrict__ hi, const float* __restrict__ lo,
                                                     double sigma, double alpha, const double* __restrict__ x,
                                                     double beta, double* __restrict__ y) {
@@ -257,10 +274,23 @@ __global__ void __launch_bounds__(kHiloThreads) k_spmv_hilo(int64_t n, int k, co
     for (int q = 0; q < Q; q++) {
         acc[q] = w0 * xi[q];
     }
-    add_slots<Q, 0>(k, col + cb, x, acc, [&](int s) {
+    // the compiler's unrolling, with wide loads of x only for eight vectors (100,003 rows,
+    // K = 30, four: 32.7 us without, 33.4 with)
+#pragma unroll 4
+    for (int s = 0; s < k; s++) {
+        const int64_t j = ld_stream(col + cb + (int64_t)s * kSlice);
         const int64_t e = vb + (int64_t)(s + 1) * kSlice;
-        return (double)ld_stream(hi + e) + (double)ld_stream(lo + e);
-    });
+        const double w = (double)ld_stream(hi + e) + (double)ld_stream(lo + e);
+        double xj[Q];
+        if constexpr (Q == 8) {
+            load_x<Q>(x, j, xj);
+        } else {
+#pragma unroll
+            for (int q = 0; q < Q; q++) xj[q] = x[j * Q + q];
+        }
+#pragma unroll
+        for (int q = 0; q < Q; q++) acc[q] = fma(w, xj[q], acc[q]);
+    }
 #pragma unroll
     for (int q = 0; q < Q; q++) {
         double out = alpha * (sigma * xi[q] - acc[q]);
@@ -272,8 +302,8 @@ __global__ void __launch_bounds__(kHiloThreads) k_spmv_hilo(int64_t n, int k, co
 template <int Q>
 mvgd_status launch_hilo(const mvgd_ell* L, double sigma, double alpha, const void* x, double beta, void* y,
                         cudaStream_t s) {
-    const unsigned blocks = (unsigned)((L->n + kHiloThreads - 1) / kHiloThreads);
-    k_spmv_hilo<Q><<<blocks, kHiloThreads, 0, s>>>(L->n, L->k, L->col, static_cast<const float*>(L->val), L->val_lo,
+    const unsigned blocks = (unsigned)((L->n + kF64Threads - 1) / kF64Threads);
+    k_spmv_hilo<Q><<<blocks, kF64Threads, 0, s>>>(L->n, L->k, L->col, static_cast<const float*>(L->val), L->val_lo,
                                           sigma, alpha, static_cast<const double*>(x), beta,
                                           static_cast<double*>(y));
     return launch_status();
