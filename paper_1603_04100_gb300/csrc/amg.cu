@@ -972,8 +972,12 @@ MVGD_API mvgd_status mvgd_amg_apply(const void* amg_ws, int64_t n, int32_t nrhs,
     cudaStream_t s = (cudaStream_t)stream;
     const int m = nlev - 1;
     if (m > 0) k_vpre<<<grid_for(n * nrhs), 256, 0, s>>>(H, b, nrhs, V.y[0]);
-    for (int l = 0; l < m; l++) k_vdown<<<grid_for(n_padded(sizes[l])), kApplyThreads, 0, s>>>(H, l, b, nrhs, V);
+    // a block for every kApplyThreads lanes of a level, kApplyThreads / G rows: by its rows
+    // alone a level of 876 rows (32 lanes each) had 4 blocks for 110 blocks' work, and each
+    // of its steps took microseconds a right-hand side
+    auto blocks = [&](int l) { return grid_for(sizes[l] * (l == 0 ? 1 : amg_group(sizes[l]))); };
+    for (int l = 0; l < m; l++) k_vdown<<<blocks(l), kApplyThreads, 0, s>>>(H, l, b, nrhs, V);
     k_vcoarse<<<grid_for(sizes[m] * kWarp), 256, 0, s>>>(H, b, x, nrhs, V);
-    for (int l = m - 1; l >= 0; l--) k_vup<<<grid_for(n_padded(sizes[l])), kApplyThreads, 0, s>>>(H, l, x, nrhs, V);
+    for (int l = m - 1; l >= 0; l--) k_vup<<<blocks(l), kApplyThreads, 0, s>>>(H, l, x, nrhs, V);
     return launch_status();
 }
