@@ -459,6 +459,14 @@ __device__ __forceinline__ bool solve6_refined(const df (&G)[21], const float (&
 // Stored row `row` of one cloud's operator in the FP32_REFINE format by the
 // FP32 path, by this lane.  Returns false (having written nothing) when the
 // row must be assembled by the FP64 path instead.
+// QUARTER: the quarter-range rule, whose h is an extent along the frame's axes
+// and so takes the frame's and the projections' errors to first order (a mean
+// distance does not see them): its barycenter, covariance and projections on
+// the tangent axes keep sums normalised at every term, of pairs rounded to
+// nearest.  99 % of the h of 30,000 points on a sphere, K = 20 and 31, come
+// out within 6.7e-15 and 8.0e-15 of FP64's (1.0e-14 and 1.2e-14 with sums
+// normalised once).
+template <bool QUARTER>
 __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) {
     extern __shared__ float smf[];
     const int lane = threadIdx.x & (kWarp - 1);
@@ -472,32 +480,50 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
 
     // offsets d_s = p_j - p_i (FP64, then double-float), barycenter of N(i),
     // mean distance to the delta_m nearest
-    df_acc sx = acc_zero(), sy = acc_zero(), sz = acc_zero(), hs = acc_zero();
+    using Sum = typename std::conditional<QUARTER, df, df_acc>::type;
+    auto sum_add = [](Sum& t, df a) {
+        if constexpr (QUARTER) t = df_add(t, a);
+        else acc_add(t, a);
+    };
+    auto sum_fma = [](Sum& t, df a, df b) {
+        if constexpr (QUARTER) t = df_fma(t, a, b);
+        else acc_fma(t, a, b);
+    };
+    auto sum_value = [](Sum t) -> df {
+        if constexpr (QUARTER) return t;
+        else return acc_value(t);
+    };
+    auto pair = [](double x) -> df {
+        if constexpr (QUARTER) return df_split_rn(x);
+        else return df_split(x);
+    };
+    Sum sx = {0.0f, 0.0f}, sy = sx, sz = sx;
+    df_acc hs = acc_zero();
     for (int s = 0; s < k; s++) {
         const int64_t j = nb[s];
         if (j < 0 || j >= A.n) return false;  // the FP64 path marks the row
-        const df dx = df_split(A.pts[3 * j] - px), dy = df_split(A.pts[3 * j + 1] - py),
-                 dz = df_split(A.pts[3 * j + 2] - pz);
+        const df dx = pair(A.pts[3 * j] - px), dy = pair(A.pts[3 * j + 1] - py),
+                 dz = pair(A.pts[3 * j + 2] - pz);
         MF(s, 0) = dx.hi; MF(s, 1) = dx.lo;
         MF(s, 2) = dy.hi; MF(s, 3) = dy.lo;
         MF(s, 4) = dz.hi; MF(s, 5) = dz.lo;
-        acc_add(sx, dx); acc_add(sy, dy); acc_add(sz, dz);
+        sum_add(sx, dx); sum_add(sy, dy); sum_add(sz, dz);
         if (s < A.delta_m) acc_add(hs, df_sqrt(df_dot3(dx, dx, dy, dy, dz, dz)));
     }
     const df kk = df_make((float)k), hsum = acc_value(hs);
-    const df cx = df_div(acc_value(sx), kk), cy = df_div(acc_value(sy), kk), cz = df_div(acc_value(sz), kk);
-    df_acc C00 = acc_zero(), C01 = C00, C02 = C00, C11 = C00, C12 = C00, C22 = C00;
+    const df cx = df_div(sum_value(sx), kk), cy = df_div(sum_value(sy), kk), cz = df_div(sum_value(sz), kk);
+    Sum C00 = {0.0f, 0.0f}, C01 = C00, C02 = C00, C11 = C00, C12 = C00, C22 = C00;
     for (int s = 0; s < k; s++) {
         const df ex = df_sub({MF(s, 0), MF(s, 1)}, cx), ey = df_sub({MF(s, 2), MF(s, 3)}, cy),
                  ez = df_sub({MF(s, 4), MF(s, 5)}, cz);
-        acc_fma(C00, ex, ex); acc_fma(C01, ex, ey); acc_fma(C02, ex, ez);
-        acc_fma(C11, ey, ey); acc_fma(C12, ey, ez); acc_fma(C22, ez, ez);
+        sum_fma(C00, ex, ex); sum_fma(C01, ex, ey); sum_fma(C02, ex, ez);
+        sum_fma(C11, ey, ey); sum_fma(C12, ey, ez); sum_fma(C22, ez, ez);
     }
 
     // frame, in FP64 (the eigen step the mixed format keeps there)
     double E[3][3], ev[3];
     {
-        auto full = [](df_acc t) { return (double)t.hi + (double)t.lo; };
+        auto full = [](Sum t) { return (double)t.hi + (double)t.lo; };
         double C[3][3] = {{full(C00), full(C01), full(C02)}, {0.0, full(C11), full(C12)}, {0.0, 0.0, full(C22)}};
         eig3(C, E, ev);
     }
@@ -508,21 +534,24 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
     }
     if (imax == imin) imin = (imax + 1) % 3;
     const int imid = 3 - imax - imin;
-    const df ex0 = df_split(E[0][imax]), ex1 = df_split(E[1][imax]), ex2 = df_split(E[2][imax]);
-    const df ey0 = df_split(E[0][imid]), ey1 = df_split(E[1][imid]), ey2 = df_split(E[2][imid]);
-    const df ez0 = df_split(E[0][imin]), ez1 = df_split(E[1][imin]), ez2 = df_split(E[2][imin]);
+    const df ex0 = pair(E[0][imax]), ex1 = pair(E[1][imax]), ex2 = pair(E[2][imax]);
+    const df ey0 = pair(E[0][imid]), ey1 = pair(E[1][imid]), ey2 = pair(E[2][imid]);
+    const df ez0 = pair(E[0][imin]), ez1 = pair(E[1][imin]), ez2 = pair(E[2][imin]);
 
     // local coordinates centred at p_i; quarter-range extents
     df x0 = df_make(3e38f), x1 = df_make(-3e38f), y0 = x0, y1 = x1;
     for (int s = 0; s < k; s++) {
         const df dx = {MF(s, 0), MF(s, 1)}, dy = {MF(s, 2), MF(s, 3)}, dz = {MF(s, 4), MF(s, 5)};
-        const df lx = df_dot3(dx, ex0, dy, ex1, dz, ex2);
-        const df ly = df_dot3(dx, ey0, dy, ey1, dz, ey2);
+        auto along = [&](df e0, df e1, df e2) {
+            if constexpr (QUARTER) return df_add(df_add(df_mul(dx, e0), df_mul(dy, e1)), df_mul(dz, e2));
+            else return df_dot3(dx, e0, dy, e1, dz, e2);
+        };
+        const df lx = along(ex0, ex1, ex2), ly = along(ey0, ey1, ey2);
         const df lz = df_dot3(dx, ez0, dy, ez1, dz, ez2);
         MF(s, 0) = lx.hi; MF(s, 1) = lx.lo;
         MF(s, 2) = ly.hi; MF(s, 3) = ly.lo;
         MF(s, 4) = lz.hi; MF(s, 5) = lz.lo;
-        if (A.delta_kind == MVGD_DELTA_QUARTER_RANGE) {
+        if constexpr (QUARTER) {
             if (df_less(lx, x0)) x0 = lx;
             if (df_less(x1, lx)) x1 = lx;
             if (df_less(ly, y0)) y0 = ly;
@@ -530,7 +559,7 @@ __device__ __noinline__ bool assemble_lane_mixed(const AsmArgs& A, int64_t row) 
         }
     }
     df h;
-    if (A.delta_kind == MVGD_DELTA_QUARTER_RANGE) {
+    if constexpr (QUARTER) {
         const df rx = df_mul_f(df_sub(x1, x0), 0.25f), ry = df_mul_f(df_sub(y1, y0), 0.25f);
         h = df_less(rx, ry) ? rx : ry;
     } else {
@@ -653,7 +682,9 @@ __device__ __forceinline__ void assemble_row(const AsmArgs& A, int64_t row, int 
         return;
     }
     if (MODE == 1 || (MODE == 2 && A.prec == MVGD_FP32_REFINE && !A.arith)) {
-        if (!assemble_lane_mixed(A, row)) {
+        const bool done = A.delta_kind == MVGD_DELTA_QUARTER_RANGE ? assemble_lane_mixed<true>(A, row)
+                                                                   : assemble_lane_mixed<false>(A, row);
+        if (!done) {
             const int pos = atomicAdd(A.nfix, 1);
             A.fix[pos] = make_int2(item, (int)row);
         }
