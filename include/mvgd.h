@@ -580,7 +580,8 @@ mvgd_status mvgd_test_withhold_arrival(int32_t on);
  *   solver_blocks_per_sm: resident blocks per SM of the persistent solver
  *     (0: as many as fit, the default; otherwise at most that many);
  *   stage_buffers: operator slices a solver warp keeps in flight, 1 (default)
- *     or 2 (used only when the shared memory allows it; 0 = 1);
+ *     or 2 (used by launches of one request, when the shared memory allows
+ *     it; 0 = 1);
  *   assemble_warps: warps per block of the FP32 assembly path, 1 (default),
  *     2, 4 or 8 (fewer when the shared memory would not fit; 0 = 1); the FP64
  *     arithmetic always takes one.

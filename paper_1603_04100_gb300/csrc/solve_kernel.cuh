@@ -1721,9 +1721,15 @@ static_assert(stage_bytes_per_warp<double>(kMaxK) * (kThreads / kWarp) <= kStage
 // rows, K = 20, three single-buffered blocks ran the FP32 multigrid solve 8 %
 // faster than two double-buffered ones (every step that is not a product
 // loses the third block's latency hiding).  mvgd_set_launch_tuning selects two.
-template <typename VT>
+// With several requests it is one whatever is selected: their steps ask for
+// nothing ahead, and a second buffer would only take its block (4 requests of
+// 200,000 rows, FP32: 32.6 ms a batch with one, 38.5 with an idle second one,
+// 37.9 with the request's next tile asked for ahead, whose code also cost the
+// launches with one buffer 1 %).
+template <typename VT, int SHARING>
 int stage_buffers(int kmax) {
-    if (tuned_stage_buffers() == 2 && 2 * stage_bytes_per_warp<VT>(kmax) * (kThreads / kWarp) <= kStageMax)
+    if (SHARING != S_LISTED && tuned_stage_buffers() == 2 &&
+        2 * stage_bytes_per_warp<VT>(kmax) * (kThreads / kWarp) <= kStageMax)
         return 2;
     return 1;
 }
@@ -1733,7 +1739,7 @@ template <bool MIXED, int QT, bool AMG, int SHARING>
 int solve_capacity(int kmax, size_t* smem_out = nullptr, size_t more = 0) {
     using VT = typename std::conditional<MIXED, float, double>::type;
     auto fn = k_solve<MIXED, QT, AMG, SHARING>;
-    const size_t smem = stage_bytes_per_warp<VT>(kmax) * (kThreads / kWarp) * stage_buffers<VT>(kmax) + more;
+    const size_t smem = stage_bytes_per_warp<VT>(kmax) * (kThreads / kWarp) * stage_buffers<VT, SHARING>(kmax) + more;
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -1764,7 +1770,7 @@ mvgd_status launch_solve_as(const ReqTable& tab, Ctl ctl, int budget, int kmax, 
     units *= tab.groups;
     if (grid > units) grid = units;
     grid -= grid % tab.groups;  // units is a multiple of groups, and groups <= 8 blocks always fit
-    int nbuf = stage_buffers<VT>(kmax);
+    int nbuf = stage_buffers<VT, SHARING>(kmax);
     ReqTable t = tab;
     void* args[] = {(void*)&t, (void*)&ctl, (void*)&budget, (void*)&kmax, (void*)&nbuf};
     MVGD_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_solve<MIXED, QT, AMG, SHARING>, dim3(grid), dim3(kThreads), args,
