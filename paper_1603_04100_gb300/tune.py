@@ -9,8 +9,10 @@ runs but never what it computes:
     persistent solver (its reductions run over fixed chunks whatever the grid);
 and keeps the fastest setting of each, one knob at a time in that order.  The
 choice is cached in a JSON file keyed by (GPU name, N rounded to a power of
-two, K, precision, preconditioner): a later run of the same shape applies it
-without searching.  Cache file: $MVGD_TUNE_CACHE, else
+two, K, precision, preconditioner, the library's bytes): a later run of the
+same shape with the same library applies it without searching.  (What was
+fastest with other kernels, or as a multiple of another cell estimate, need
+not be now.)  Cache file: $MVGD_TUNE_CACHE, else
 ~/.cache/mvgd_gb300/tune.json.
 
     tuning = tune_pipeline(pipe, pts, f)   # times, caches, applies
@@ -19,6 +21,8 @@ without searching.  Cache file: $MVGD_TUNE_CACHE, else
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import math
 import os
@@ -29,6 +33,7 @@ from pathlib import Path
 import torch
 
 from . import _lib as LB
+from . import build
 
 CELL_FACTORS = (0.7, 0.85, 1.0, 1.2, 1.45)
 ASSEMBLE_WARPS = (1, 2, 4)
@@ -58,9 +63,22 @@ def cache_path() -> Path:
     return Path(env) if env else Path.home() / ".cache" / "mvgd_gb300" / "tune.json"
 
 
+@functools.lru_cache(maxsize=None)
+def _library_id(path: str, size: int, mtime_ns: int) -> str:
+    return hashlib.sha256(Path(path).read_bytes()).hexdigest()[:12]
+
+
+def library_id() -> str:
+    """The built library, by its bytes ("none" before the first build)."""
+    if not build.LIB.exists():
+        return "none"
+    st = build.LIB.stat()
+    return _library_id(str(build.LIB), st.st_size, st.st_mtime_ns)
+
+
 def shape_key(n: int, k: int, prec: int, precond: int, device=None) -> str:
     name = torch.cuda.get_device_name(device) if torch.cuda.is_available() else "cpu"
-    return f"{name}|n2^{round(math.log2(max(n, 2)))}|k{k}|prec{prec}|precond{precond}"
+    return f"{name}|n2^{round(math.log2(max(n, 2)))}|k{k}|prec{prec}|precond{precond}|lib{library_id()}"
 
 
 def load_cache(path: Path | None = None) -> dict:
