@@ -135,7 +135,10 @@ __global__ void k_neumann_flags(const uint8_t* __restrict__ boundary, const int3
         const bool bnd = boundary[i] != 0;
         bool near = false;
         if (!bnd)
-            for (int s = 0; s < k; s++) near |= boundary[nbr[i * k + s]] != 0;
+            for (int s = 0; s < k; s++) {  // (-1: a cloud without a finite extent has no lists)
+                const int32_t j = nbr[i * k + s];
+                near |= j >= 0 && j < n && boundary[j] != 0;
+            }
         fi[i] = bnd ? 0 : 1;
         fb[i] = bnd ? 1 : 0;
         fm[i] = near ? 1 : 0;
@@ -183,7 +186,7 @@ __device__ void covariance(const double (*d)[3], int cnt, double C[3][3]) {
 }
 
 // e3 of every boundary point (one thread each); bad frames counted in *bad.
-__global__ void k_boundary_frames(const double* __restrict__ pts, const int32_t* __restrict__ nbr, int k,
+__global__ void k_boundary_frames(const double* __restrict__ pts, int64_t n, const int32_t* __restrict__ nbr, int k,
                                   const int32_t* __restrict__ bidx, const int32_t* __restrict__ nb_ptr, int kb,
                                   double* __restrict__ e3, int32_t* __restrict__ bad) {
     const int nb = *nb_ptr;
@@ -194,8 +197,14 @@ __global__ void k_boundary_frames(const double* __restrict__ pts, const int32_t*
     double d[kMaxK > kMaxKb ? kMaxK + 1 : kMaxKb + 1][3];
     double C[3][3], V[3][3], w[3];
     // e2: the surface normal from the K neighbours in the whole cloud
+    bool listed = true;
     for (int s = 0; s < k; s++) {
-        const double* Q = pts + 3 * (int64_t)nbr[ib * k + s];
+        int64_t j = nbr[ib * k + s];
+        if (j < 0 || j >= n) {
+            listed = false;
+            j = ib;
+        }
+        const double* Q = pts + 3 * j;
         for (int c = 0; c < 3; c++) d[s][c] = Q[c] - P[c];
     }
     covariance(d, k, C);
@@ -221,7 +230,7 @@ __global__ void k_boundary_frames(const double* __restrict__ pts, const int32_t*
         bd[at] = dd;
         bi[at] = ic;
     }
-    bool ok = kbe >= 2;
+    bool ok = kbe >= 2 && listed;
     double out[3] = {0.0, 0.0, 0.0};
     if (ok) {
         // principal axis t and the other two axes u, v of p_b and its boundary neighbours
@@ -508,7 +517,7 @@ MVGD_API mvgd_status mvgd_neumann_ghosts(const double* pts, int64_t n, int32_t k
     scan_flags(fm, n, pos_g, tiles, cnt + 2, s);
     k_neumann_compact<<<g, 256, 0, s>>>(pts, n, fi, pos_i, pos_b, q, q_src, interior, bidx);
     // one thread per boundary point; launched for n (the count is on the device)
-    k_boundary_frames<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(pts, nbr, k, bidx, cnt + 1, kb, e3, cnt + 3);
+    k_boundary_frames<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(pts, n, nbr, k, bidx, cnt + 1, kb, e3, cnt + 3);
     // the caller's counts: interior points, ghosts, boundary points, bad frames
     k_neumann_counts<<<1, 32, 0, s>>>(cnt, counts);
     k_ghosts<<<g, 256, 0, s>>>(pts, n, fm, pos_i, pos_g, bidx, counts, e3, q, q_src, ghost_bnd, ghost_dist);
