@@ -436,7 +436,8 @@ mvgd_status mvgd_solve(const mvgd_ell *L, int32_t nrhs, double sigma, const doub
  *     kept as FP32 for the cycle);
  *   - the first level with <= MVGD_AMG_COARSEST rows is inverted
  *     (Gauss-Jordan with partial pivoting in FP32, then two Newton-Schulz
- *     steps in FP64) and solved by an FP64 product with that inverse;
+ *     steps: the last residual in FP64, the corrections on hi + lo FP32
+ *     words) and solved by an FP64 product with that inverse;
  *   - one V(1,1)-cycle in FP32 with Jacobi smoothing x += d (b - A x):
  *     d_i = MVGD_AMG_JACOBI_OMEGA / a_ii on rows with a strong diagonal
  *     (a_ii > MVGD_AMG_JACOBI_THETA sum_j |a_ij|), the l1 scaling

@@ -654,7 +654,10 @@ __global__ void __launch_bounds__(kInvThreads) k_amg_invert(AmgHeader* Hp) {
 // A block of 4 warps takes a 16 x 16 tile (256 tiles at n = 256: more than SMs);
 // each warp takes every fourth group of 8 of the sum, 8 outputs a lane, and the
 // block adds the four partial sums.  All four: 317 -> 98 us at n = 256, of which
-// R1 43 us (27 at the FP64 pipe's rate).
+// R1 43 us (27 at the FP64 pipe's rate).  Against 80-bit arithmetic, with all four
+// in FP64 before: the residual I - A X 0.07 to 0.16 of it, the error of X 0.68
+// (300 rows of a one-level hierarchy) and 1.2 (Galerkin levels of 110 to 469 rows,
+// from the order of R1's sums; the splits add nothing).
 // ---------------------------------------------------------------------------
 enum NsStep : int { kNsR0 = 0, kNsX1 = 1, kNsR1 = 2, kNsX2 = 3 };
 constexpr int kNsTile = 16, kNsDeep = 32, kNsWarps = 4;

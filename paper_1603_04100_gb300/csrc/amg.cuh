@@ -48,7 +48,8 @@ struct AmgHeader {
     int32_t prec0, pad0;
     float* cinv;        // [nc][nc] its FP32 Gauss-Jordan inverse, column-major: cinv[c * nc + r] = (A_c^-1)[r][c]
     double* dense64;    // [nc][nc] the coarsest level, FP64 row-major
-    double* cinv64;     // [nc][nc] the inverse after two Newton-Schulz steps in FP64, row-major (what the cycle uses)
+    double* cinv64;     // [nc][nc] the inverse after two Newton-Schulz steps (the last residual in FP64, see
+                        //   amg.cu), row-major: what the cycle uses
     double* ns_x;       // [nc][nc] set-up scratch
     double* ns_t;       // [nc][nc] set-up scratch
     float* ns_s;        // [nc][nc][2] set-up scratch

@@ -105,15 +105,14 @@ __device__ __forceinline__ float jacobi_tan(float apq, float d) {
 // Eigenvectors (columns of e) of a symmetric 3x3 matrix to FP64 accuracy, w the
 // eigenvalues (for their order; c is overwritten).  A plain FP64 Jacobi takes five
 // or six sweeps and spends most of their instructions in divisions and square
-// roots on the FP64 pipe (one instruction in 16 clocks a warp): some 1,150 of
-// them.  Here the sweeps that only find the frame run in FP32; its vectors are
-// orthonormalised in FP64, the matrix is rotated into them, and FP64 rotations
-// finish.  A rotation need not annihilate exactly, it must only be orthogonal:
-// its tangent comes from FP32, its cosine from an FP32 root with one cubic Newton
-// step, so an off-diagonal entry shrinks by 1e-7 a sweep beside Jacobi's own
-// quadratic rate.  Once the remaining angles are below 2^-27 one first-order
-// update is exact to rounding.  About 330 FP64 instructions, of general inputs:
-// the entries are scaled by a power of two first.
+// roots on the FP64 pipe (one instruction in 16 clocks a warp).  Here the sweeps
+// that only find the frame run in FP32; its vectors are orthonormalised in FP64,
+// the matrix is rotated into them, and FP64 rotations finish.  A rotation need
+// not annihilate exactly, it must only be orthogonal: its tangent comes from FP32,
+// its cosine from an FP32 root with one cubic Newton step, so an off-diagonal entry
+// shrinks by 1e-7 a sweep beside Jacobi's own quadratic rate.  Once the remaining angles are below 2^-27 one first-order
+// update is exact to about 2^-49 of a radian.  For general inputs the entries are
+// scaled by a power of two first.
 __device__ inline void eig3(double (&c)[3][3], double (&e)[3][3], double (&w)[3]) {
     {
         const double m = fmax(fabs(c[0][0]), fmax(fabs(c[1][1]), fabs(c[2][2])));

